@@ -38,6 +38,13 @@ constexpr uint32_t kLzLenRing = 512;   // pre-parsed lengths per warp
 constexpr uint32_t kLzBatch = 480;     // lengths parsed ahead per refill (at most ring - 32)
 constexpr uint32_t kLzWin = 4096;      // batch output window per warp
 constexpr uint32_t kFull = 0xFFFFFFFFu;
+// Launches of at most this many blocks per SM take a CTA per block
+// (zf_lz_cta.cu).  A warp takes 540 us for a block of text however few there
+// are, a CTA per block adds 0.32 us for each block to about 60 us: resident
+// calls of 8, 64, 128 and 160 MB took 100, 387, 726 and 870 us with a CTA and
+// 568, 681, 791 and 848 us with a warp per block (2,432 blocks, 16 per SM,
+// would be even).
+constexpr uint32_t kLzCtaBlocksPerSm = 14;
 
 struct LzParse {
     uint32_t vp = 0;        // next byte of the lengths stream
@@ -331,6 +338,7 @@ namespace zf {
 
 cudaError_t launch_lz(const ZfDevChunk* chunks, uint32_t n, uint32_t* err, int num_sms, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
+    if (n <= (uint32_t)num_sms * kLzCtaBlocksPerSm) return launch_lz_cta(chunks, n, err, s);
     // one warp (one block) per CTA, so a small launch still spreads over
     // every SM; up to 32 CTAs per SM, then warps loop over the rest
     uint32_t blocks = n;
