@@ -143,7 +143,8 @@ typedef struct {
 typedef struct {
     uint32_t tile_rows;       /* rows per warp job: a multiple of 1024, <= 16384 (0 = the
                                  class's tuned value, else 2048 for delta launches
-                                 and 4096 for the others) */
+                                 and 4096 for the others, halved down to 1024 while
+                                 a launch has fewer than 32 jobs per SM) */
     uint32_t threads;         /* 128, 256 or 512 (0 = the class's tuned value, else 128) */
     uint32_t ctas_per_sm;     /* batched launch: persistent grid = ctas_per_sm x SM count (0 = occupancy limit) */
     uint32_t stage_bytes;     /* pipeline stage: compressed bytes per H2D copy + decode step (default 64 MiB) */

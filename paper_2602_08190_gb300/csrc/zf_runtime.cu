@@ -124,14 +124,23 @@ uint32_t width_bucket(uint32_t bmax) { return bmax <= 8 ? 0u : bmax <= 16 ? 1u :
 struct Geometry {
     uint32_t tile_rows, threads;
 };
-Geometry group_geometry(const zf_ctx* ctx, const zf_kcfg& k, int scheme, int dtype, uint32_t bmax) {
+// The built-in job is halved while the launch's `units` (rows or tokens) would
+// give an SM fewer than 32 warps: a job's tiles follow one another, so in a
+// launch that leaves warps idle every tile but the first only waits (a
+// resident call of 1M rows took 24.4, 30.4 and 38.1 us as FOR, RLE and
+// Float2Int and takes 22.6, 23.6 and 25.6 us; 4 MB of string dictionary 107
+// and 71 us; from 32M rows on nothing changes).  units = 0: not known.
+Geometry group_geometry(const zf_ctx* ctx, const zf_kcfg& k, int scheme, int dtype, uint32_t bmax, uint64_t units) {
     Geometry g{k.tile_rows, k.threads};
     if (scheme >= 0 && scheme < ZF_NSCHEMES && dtype >= 0 && dtype < 4) {
         const auto& t = ctx->tuned[scheme][dtype][width_bucket(bmax)];
         if (!g.tile_rows) g.tile_rows = t.tile_rows;
         if (!g.threads) g.threads = t.threads;
     }
-    if (!g.tile_rows) g.tile_rows = scheme == ZF_DELTA_BP ? 2048u : 4096u;
+    if (!g.tile_rows) {
+        g.tile_rows = scheme == ZF_DELTA_BP ? 2048u : 4096u;
+        while (units && g.tile_rows > 1024 && units < (uint64_t)g.tile_rows * 32u * ctx->num_sms) g.tile_rows /= 2;
+    }
     if (!g.threads) g.threads = 128;
     return g;
 }
@@ -256,9 +265,14 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
     }
     for (auto& key : keys) {
         uint32_t bmax = 0;   // widest bit width of the group: its geometry class
-        for (size_t i = b; i < e; i++)
-            if (w[i].ch->scheme == key.first && w[i].ch->dtype == key.second) bmax = std::max<uint32_t>(bmax, w[i].ch->bmax);
-        const Geometry geo = group_geometry(ctx, k, key.first, key.second, bmax);
+        uint64_t units = 0;  // rows (string dictionary: tokens) of the group
+        for (size_t i = b; i < e; i++) {
+            const zf::ChunkInfo& ch = *w[i].ch;
+            if (ch.scheme == key.first && ch.dtype == key.second) bmax = std::max<uint32_t>(bmax, ch.bmax);
+            if (key.first < 0 ? ch.scheme != ZF_LZ77 && ch.scheme != ZF_ANS : ch.scheme == key.first && ch.dtype == key.second)
+                units += ch.scheme == ZF_STRDICT ? ch.units : ch.rows;
+        }
+        const Geometry geo = group_geometry(ctx, k, key.first, key.second, bmax, units);
         Group g{key.first, key.second, (uint32_t)desc.size(), 0, 0, 16, geo.tile_rows, geo.threads};
         for (size_t i = b; i < e; i++) {
             int s = w[i].ch->scheme, d = w[i].ch->dtype;
@@ -1297,7 +1311,7 @@ extern "C" zf_status zf_ctx_tuned_geometry(const zf_ctx* ctx, int32_t scheme, in
     if (!ctx || !out || scheme < 0 || scheme >= ZF_NSCHEMES || dtype < 0 || dtype > ZF_F64 || bmax > 64)
         return ZF_EINVAL;
     const zf_kcfg k = effective_kcfg(ctx);
-    const Geometry g = group_geometry(ctx, k, scheme, dtype, bmax);
+    const Geometry g = group_geometry(ctx, k, scheme, dtype, bmax, 0);
     *out = k;
     out->tile_rows = g.tile_rows;
     out->threads = g.threads;
