@@ -146,16 +146,17 @@ __device__ __forceinline__ bool ans_stream(const AnsSmem& sm, const uint8_t* s2,
 
 // The CTA builds its chunk's tables, then warp w decodes job blockIdx.x *
 // kWarps + w: lane i takes the job's stream i.
-__global__ void __launch_bounds__(kWarps * 32) ans_kernel(const ZfDevChunk* chunks, uint32_t nchunks, uint32_t njobs,
+__global__ void __launch_bounds__(kWarps * 32) ans_kernel(const __grid_constant__ zf::ChunkArgs args, uint32_t njobs,
                                                            uint32_t* err) {
     __shared__ AnsSmem sm;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t job0 = blockIdx.x * kWarps;
     if (job0 >= njobs) return;
-    uint32_t a = 0, z = nchunks;
+    const ZfDevChunk* chunks = args.list();
+    uint32_t a = 0, z = args.n;
     while (z - a > 1) {
         const uint32_t mid = (a + z) >> 1;
-        if (__ldg(&chunks[mid].tile0) <= job0) a = mid;
+        if (chunks[mid].tile0 <= job0) a = mid;
         else z = mid;
     }
     const ZfDevChunk c = chunks[a];
@@ -252,9 +253,10 @@ __global__ void __launch_bounds__(kWarps * 32) ans_kernel(const ZfDevChunk* chun
 namespace zf {
 
 // njobs is a multiple of kAnsJobsPerCta: every chunk's jobs are padded to it.
-cudaError_t launch_ans(const ZfDevChunk* chunks, uint32_t nchunks, uint32_t njobs, uint32_t* err, cudaStream_t s) {
+cudaError_t launch_ans(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t nchunks, uint32_t njobs, uint32_t* err,
+                       cudaStream_t s) {
     if (njobs == 0) return cudaSuccess;
-    ans_kernel<<<(njobs + kWarps - 1) / kWarps, kWarps * 32, 0, s>>>(chunks, nchunks, njobs, err);
+    ans_kernel<<<(njobs + kWarps - 1) / kWarps, kWarps * 32, 0, s>>>(ChunkArgs(chunks, host, nchunks), njobs, err);
     return cudaGetLastError();
 }
 

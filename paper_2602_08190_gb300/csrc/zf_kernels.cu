@@ -19,8 +19,7 @@
 namespace {
 
 struct LaunchArgs {
-    const ZfDevChunk* chunks;
-    uint32_t nchunks;
+    zf::ChunkArgs chunks;
     uint32_t njobs;        // warp jobs in the launch
     uint32_t job_rows;     // rows of one warp job (a multiple of 1024)
     uint32_t warp_smem;    // bytes of shared memory per warp
@@ -59,7 +58,7 @@ __device__ __forceinline__ uint32_t find_chunk(const ZfDevChunk* ch, uint32_t n,
     uint32_t a = 0, z = n;
     while (z - a > 1) {
         uint32_t mid = (a + z) >> 1;
-        if (__ldg(&ch[mid].tile0) <= job) a = mid;
+        if (ch[mid].tile0 <= job) a = mid;
         else z = mid;
     }
     return a;
@@ -116,8 +115,8 @@ __device__ __forceinline__ void decode_mixed(const ZfDevChunk& c, const zfd::Hdr
 // chunk may be shorter).
 template <int SCHEME, int DT>
 __device__ __forceinline__ void run_job(const LaunchArgs& a, uint32_t job, uint32_t* wsm) {
-    const uint32_t k = find_chunk(a.chunks, a.nchunks, job);
-    const ZfDevChunk c = a.chunks[k];
+    const ZfDevChunk* chunks = a.chunks.list();
+    const ZfDevChunk c = chunks[find_chunk(chunks, a.chunks.n, job)];
     zfd::Hdr h;
     zfd::load_hdr(c.blob, h);
     const uint32_t r0 = (job - c.tile0) * a.job_rows;
@@ -137,7 +136,7 @@ __device__ __forceinline__ void run_job(const LaunchArgs& a, uint32_t job, uint3
 // the launch can be replayed from a CUDA graph.
 // At least 32 resident warps per SM: registers are capped at 64 per thread.
 template <int SCHEME, int DT, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) tiles_kernel(LaunchArgs a) {
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) tiles_kernel(const __grid_constant__ LaunchArgs a) {
     extern __shared__ uint4 smem4[];
     constexpr uint32_t NW = THREADS / 32;
     const uint32_t warp = threadIdx.x >> 5;
@@ -185,7 +184,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) tiles_kernel(LaunchAr
 }
 
 // ---------------------------------------------------------------- launch table
-typedef void (*KernelFn)(LaunchArgs);
+typedef void (*KernelFn)(const LaunchArgs);
 
 template <int THREADS>
 KernelFn pick(int scheme, int dtype) {
@@ -267,7 +266,7 @@ cudaError_t launch_tiles(const TileLaunch& L, cudaStream_t s) {
     }
     if (grid == 0) return cudaSuccess;
     const bool affinity = L.scheme == ZF_STRDICT && L.num_sms > 0 && L.num_sms <= (int)kAffinitySms;
-    LaunchArgs a{L.chunks, L.nchunks, L.ntiles, L.tile_rows, L.smem / nw, L.err,
+    const LaunchArgs a{zf::ChunkArgs(L.chunks, L.host, L.nchunks), L.ntiles, L.tile_rows, L.smem / nw, L.err,
                  (L.scheme < 0 || affinity) ? L.queue : nullptr, (uint32_t)L.num_sms};
     fn<<<(unsigned)grid, L.threads, L.smem, s>>>(a);
     return cudaGetLastError();

@@ -336,9 +336,10 @@ __global__ void __launch_bounds__(32, 32) lz_kernel(const ZfDevChunk* chunks, ui
 
 namespace zf {
 
-cudaError_t launch_lz(const ZfDevChunk* chunks, uint32_t n, uint32_t* err, int num_sms, cudaStream_t s) {
+cudaError_t launch_lz(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t n, uint32_t* err, int num_sms,
+                      cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    if (n <= (uint32_t)num_sms * kLzCtaBlocksPerSm) return launch_lz_cta(chunks, n, err, s);
+    if (n <= (uint32_t)num_sms * kLzCtaBlocksPerSm || !chunks) return launch_lz_cta(ChunkArgs(chunks, host, n), err, s);
     // one warp (one block) per CTA, so a small launch still spreads over
     // every SM; up to 32 CTAs per SM, then warps loop over the rest
     uint32_t blocks = n;

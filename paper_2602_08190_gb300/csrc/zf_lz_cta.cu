@@ -341,9 +341,10 @@ __device__ void lz_block(const ZfDevChunk& c, LzSmem& sm, uint32_t* err) {
     if (__syncthreads_or(bad || !ok) && tid == 0) zfd::report(err, ZF_ECORRUPT, c.chunk_id);
 }
 
-__global__ void __launch_bounds__(kLzThreads, 2) lz_cta_kernel(const ZfDevChunk* chunks, uint32_t* err) {
+__global__ void __launch_bounds__(kLzThreads, 2) lz_cta_kernel(const __grid_constant__ zf::ChunkArgs chunks,
+                                                               uint32_t* err) {
     extern __shared__ uint4 smem4[];
-    const ZfDevChunk c = chunks[blockIdx.x];
+    const ZfDevChunk c = chunks.list()[blockIdx.x];
     lz_block(c, *reinterpret_cast<LzSmem*>(smem4), err);
 }
 
@@ -355,7 +356,7 @@ bool g_attr_set[kMaxDevices];   // shared-memory attribute of lz_cta_kernel set 
 
 namespace zf {
 
-cudaError_t launch_lz_cta(const ZfDevChunk* chunks, uint32_t n, uint32_t* err, cudaStream_t s) {
+cudaError_t launch_lz_cta(const ChunkArgs& chunks, uint32_t* err, cudaStream_t s) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -367,7 +368,7 @@ cudaError_t launch_lz_cta(const ZfDevChunk* chunks, uint32_t n, uint32_t* err, c
             if (dev < kMaxDevices) g_attr_set[dev] = true;
         }
     }
-    lz_cta_kernel<<<n, kLzThreads, sizeof(LzSmem), s>>>(chunks, err);
+    lz_cta_kernel<<<chunks.n, kLzThreads, sizeof(LzSmem), s>>>(chunks, err);
     return cudaGetLastError();
 }
 

@@ -301,18 +301,28 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
     }
 }
 
-zf_status launch_groups(zf_ctx* ctx, const std::vector<Group>& groups, const ZfDevChunk* d_desc, const zf_kcfg& k,
-                        cudaStream_t stream, uint32_t* queue) {
-    for (const Group& g : groups) {
-        const ZfDevChunk* dchunks = d_desc + g.first;
+// Whether every launch of a call takes its descriptors as parameters, so
+// that none have to be copied to the device.
+bool all_inline(const std::vector<Group>& groups) {
+    for (const Group& g : groups)
+        if (g.count > zf::kInlineChunks) return false;
+    return true;
+}
+
+// d_desc: the call's descriptors on the device, or null (all_inline); h_desc: on the host.
+zf_status launch_groups(zf_ctx* ctx, const Group* groups, size_t ngroups, const ZfDevChunk* d_desc,
+                        const ZfDevChunk* h_desc, const zf_kcfg& k, cudaStream_t stream, uint32_t* queue) {
+    for (size_t i = 0; i < ngroups; i++) {
+        const Group& g = groups[i];
+        const ZfDevChunk *dchunks = d_desc ? d_desc + g.first : nullptr, *hchunks = h_desc + g.first;
         cudaError_t e;
         if (g.scheme == ZF_LZ77) {
-            e = zf::launch_lz(dchunks, g.count, ctx->d_errw, ctx->num_sms, stream);
+            e = zf::launch_lz(dchunks, hchunks, g.count, ctx->d_errw, ctx->num_sms, stream);
         } else if (g.scheme == ZF_ANS) {
-            e = zf::launch_ans(dchunks, g.count, g.ntiles, ctx->d_errw, stream);
+            e = zf::launch_ans(dchunks, hchunks, g.count, g.ntiles, ctx->d_errw, stream);
         } else {
             uint32_t smem = ((g.warp_smem + 15) & ~15u) * (g.threads / 32);
-            zf::TileLaunch L{dchunks, g.count, g.ntiles, g.scheme, g.dtype, g.tile_rows, g.threads,
+            zf::TileLaunch L{dchunks, hchunks, g.count, g.ntiles, g.scheme, g.dtype, g.tile_rows, g.threads,
                              k.ctas_per_sm, smem, ctx->num_sms, ctx->d_errw, queue};
             e = zf::launch_tiles(L, stream);
         }
@@ -674,9 +684,12 @@ zf_status zf_transfer_decompress(zf_ctx* ctx, const zf_compressed* const* cols, 
     std::vector<std::vector<Group>> groups(stages.size());
     for (size_t s = 0; s < stages.size(); s++) build_groups(ctx, work, stages[s].first, stages[s].second, k, desc, groups[s]);
     const size_t nd = std::max<size_t>(desc.size(), 1);
-    ZfDevChunk* d_desc;
-    ZfDevChunk* h_desc;
-    if (use_graph) {
+    ZfDevChunk* d_desc = nullptr;
+    ZfDevChunk* h_desc = nullptr;
+    const bool inl = std::all_of(groups.begin(), groups.end(), all_inline);
+    if (inl) {
+        // every launch carries its descriptors: nothing to copy
+    } else if (use_graph) {
         // the graph keeps its own descriptor buffers: other calls reuse the context's
         if (nd > ctx->g_desc_cap) {
             if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
@@ -706,7 +719,7 @@ zf_status zf_transfer_decompress(zf_ctx* ctx, const zf_compressed* const* cols, 
         d_desc = ctx->d_desc;
         h_desc = ctx->h_desc;
     }
-    if (!desc.empty()) memcpy(h_desc, desc.data(), desc.size() * sizeof(ZfDevChunk));
+    if (!inl) memcpy(h_desc, desc.data(), desc.size() * sizeof(ZfDevChunk));
     if (use_graph) {
         // capture the whole call (both streams) into a graph, then launch it
         if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
@@ -737,10 +750,10 @@ zf_status zf_transfer_decompress(zf_ctx* ctx, const zf_compressed* const* cols, 
         cudaError_t e_ = (call);                                              \
         if (e_ != cudaSuccess) return abort_capture(cuda_fail(ctx, e_, #call)); \
     } while (0)
-    // the error word and the descriptors go first on the copy stream: an H2D
-    // copy on another stream can queue behind the stage copies on the same
-    // copy engine and hold every decode back
-    if (!desc.empty())
+    // the descriptors go first on the copy stream: an H2D copy on another
+    // stream can queue behind the stage copies on the same copy engine and
+    // hold every decode back
+    if (!inl)
         ZF_CAP(cudaMemcpyAsync(d_desc, h_desc, desc.size() * sizeof(ZfDevChunk), cudaMemcpyHostToDevice, ctx->copy));
     if (stages.empty()) ZF_CAP(cudaEventRecord(ctx->ev_copied[0], ctx->copy));
     if (stages.empty()) ZF_CAP(cudaStreamWaitEvent(ctx->compute, ctx->ev_copied[0], 0));
@@ -751,7 +764,8 @@ zf_status zf_transfer_decompress(zf_ctx* ctx, const zf_compressed* const* cols, 
             ZF_CAP(cudaMemcpyAsync(ctx->slots[slot] + p.slot_off, p.src, p.bytes, cudaMemcpyHostToDevice, ctx->copy));
         ZF_CAP(cudaEventRecord(ctx->ev_copied[slot], ctx->copy));
         ZF_CAP(cudaStreamWaitEvent(ctx->lane[slot], ctx->ev_copied[slot], 0));
-        st = launch_groups(ctx, groups[s], d_desc, k, ctx->lane[slot], ctx->d_err + zf::kQueueWords * slot);
+        st = launch_groups(ctx, groups[s].data(), groups[s].size(), d_desc, desc.data(), k, ctx->lane[slot],
+                           ctx->d_err + zf::kQueueWords * slot);
         if (st) return abort_capture(st);
         ZF_CAP(cudaEventRecord(ctx->ev_free[slot], ctx->lane[slot]));
     }
@@ -912,20 +926,20 @@ zf_status zf_decompress_resident(zf_ctx* ctx, const zf_resident* const* cols, ui
     std::vector<Group> groups;
     build_groups(ctx, work, 0, work.size(), k, desc, groups);
     ZF_CU(ctx, cudaEventRecord(ctx->ev_t0, ctx->compute));
-    bool same = desc.size() == ctx->resident_cache.size() &&
-                (desc.empty() || memcmp(desc.data(), ctx->resident_cache.data(), desc.size() * sizeof(ZfDevChunk)) == 0);
+    const bool inl = all_inline(groups);
+    const bool same = inl || (desc.size() == ctx->resident_cache.size() &&
+                              memcmp(desc.data(), ctx->resident_cache.data(), desc.size() * sizeof(ZfDevChunk)) == 0);
     if (!same) {
-        st = ensure_desc(ctx, std::max<size_t>(desc.size(), 1));
+        st = ensure_desc(ctx, desc.size());
         if (st) return st;
-        if (!desc.empty()) {
-            memcpy(ctx->h_desc, desc.data(), desc.size() * sizeof(ZfDevChunk));
-            ZF_CU(ctx, cudaMemcpyAsync(ctx->d_desc, ctx->h_desc, desc.size() * sizeof(ZfDevChunk),
-                                       cudaMemcpyHostToDevice, ctx->compute));
-        }
+        memcpy(ctx->h_desc, desc.data(), desc.size() * sizeof(ZfDevChunk));
+        ZF_CU(ctx, cudaMemcpyAsync(ctx->d_desc, ctx->h_desc, desc.size() * sizeof(ZfDevChunk), cudaMemcpyHostToDevice,
+                                   ctx->compute));
         ctx->resident_cache = desc;
     }
+    const ZfDevChunk* d_desc = inl ? nullptr : ctx->d_desc;
     if (groups.size() <= 1) {
-        st = launch_groups(ctx, groups, ctx->d_desc, k, ctx->compute, ctx->d_err);
+        st = launch_groups(ctx, groups.data(), groups.size(), d_desc, desc.data(), k, ctx->compute, ctx->d_err);
     } else {
         // one launch per (scheme, dtype) group, each on its own decode stream,
         // so a launch's tail overlaps the next launch's start
@@ -934,8 +948,7 @@ zf_status zf_decompress_resident(zf_ctx* ctx, const zf_resident* const* cols, ui
         for (size_t q = 0; q < nl; q++) ZF_CU(ctx, cudaStreamWaitEvent(ctx->lane[q], ctx->ev_fork, 0));
         for (size_t gi = 0; gi < groups.size() && st == ZF_OK; gi++) {
             const size_t q = gi % nl;
-            st = launch_groups(ctx, std::vector<Group>{groups[gi]}, ctx->d_desc, k, ctx->lane[q],
-                               ctx->d_err + zf::kQueueWords * q);
+            st = launch_groups(ctx, &groups[gi], 1, d_desc, desc.data(), k, ctx->lane[q], ctx->d_err + zf::kQueueWords * q);
         }
         for (size_t q = 0; q < nl; q++) {
             ZF_CU(ctx, cudaEventRecord(ctx->ev_free[q], ctx->lane[q]));
