@@ -93,7 +93,7 @@ __device__ __forceinline__ uint64_t extract(const uint32_t* sm, uint32_t bitpos,
 // it are inlined into their kernels (the batched kernel included): inside a
 // function called out of line (through the ABI) the same store was seen to
 // write only its first word on sm_103a, so no out-of-line function uses it
-// (WS = false there, as in delta_block_wide and the allocation-free kernel).
+// (WS = false in delta_block_wide).
 __device__ __forceinline__ void store32(void* dst, unsigned long long a, unsigned long long b, unsigned long long c,
                                         unsigned long long d) {
     const size_t g = __cvta_generic_to_global(dst);
@@ -535,7 +535,7 @@ __device__ __noinline__ void delta_block_wide(T* dst, const uint32_t* wsm, uint3
 // Blocks of rows [r0, r0 + nrows) (r0 a multiple of 1024, at most 32 blocks).
 // Lane j holds block j's 24-byte entry; block i+1's payload is staged while
 // block i decodes.
-template <class T, bool WS>
+template <class T>
 __device__ void delta_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t nrows, uint32_t* wsm,
                           uint32_t* err, uint32_t bmax) {
     using U = typename std::conditional<sizeof(T) == 8, unsigned long long, unsigned int>::type;
@@ -584,12 +584,10 @@ __device__ void delta_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32
         const uint32_t mk = min(zf::kDeltaBlock, nrows - i * zf::kDeltaBlock);
         if ((ok_mask >> i) & 1) {
             T* dst = reinterpret_cast<T*>(c.dst) + r0 + i * zf::kDeltaBlock;
-            const bool al32 = (reinterpret_cast<uintptr_t>(dst) & 31) == 0;
             const uint32_t* buf = wsm + (i & 1) * sb;
             uint4* xb = reinterpret_cast<uint4*>(wsm + 2 * sb);
-            if (b <= 21) delta_block_lanes<T, false, WS>(dst, buf, mk, b, base, md, lane, xb);
+            if (b <= 21) delta_block_lanes<T, false, true>(dst, buf, mk, b, base, md, lane, xb);
             else delta_block_wide<T>(dst, buf, mk, b, base, md, lane);
-            (void)al32;
         }
         __syncwarp();
     }
@@ -601,7 +599,7 @@ __device__ void delta_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32
 // memory, or in global memory when the tile has more runs than a staging
 // buffer holds), and their values at `vals`.  `bm` is the warp's 32-word
 // bitmask of the tile's rows.
-template <class T, bool WS>
+template <class T>
 __device__ __forceinline__ void rle_rows(const ZfDevChunk& c, const Hdr& h, T* dst, const uint32_t* lens_al,
                                          uint32_t sft, const T* vals, uint32_t* bm, uint32_t m, uint32_t skip,
                                          uint32_t nr, bool last_tile, uint32_t next_skip, uint32_t lane,
@@ -680,7 +678,7 @@ __device__ __forceinline__ void rle_rows(const ZfDevChunk& c, const Hdr& h, T* d
     const uint32_t cnt = __popc(word);
     const uint32_t before = warp_incl_sum<uint32_t>(cnt, lane) - cnt;
     constexpr int V = 8;
-    const bool al32 = WS && (reinterpret_cast<uintptr_t>(dst) & 31) == 0;
+    const bool al32 = (reinterpret_cast<uintptr_t>(dst) & 31) == 0;
     const uint32_t o = (lane & 3) * 8;
     for (uint32_t row = 0; row * 256 < nr; row++) {
         const uint32_t j = row * 256 + lane * V;
@@ -723,7 +721,7 @@ __host__ __device__ inline uint32_t rle_buf_bytes(uint32_t value_bytes) {
 // Tiles of rows [r0, r0 + nrows) (r0 a multiple of 1024, at most 31 tiles).
 // Lane j holds the directory entry of tile j (and of the tile after the
 // last); the next tile's lengths and values are staged while a tile expands.
-template <class T, bool WS>
+template <class T>
 __device__ void rle_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t nrows, uint32_t* wsm,
                         uint32_t* err) {
     const uint32_t lane = threadIdx.x & 31;
@@ -803,11 +801,11 @@ __device__ void rle_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t
             T* dst = reinterpret_cast<T*>(c.dst) + rr;
             if (m <= kRleStageRuns) {
                 const uint8_t* b = bufs + (i % kRleStages) * bb;
-                rle_rows<T, WS>(c, h, dst, reinterpret_cast<const uint32_t*>(b), rf & 3u,
+                rle_rows<T>(c, h, dst, reinterpret_cast<const uint32_t*>(b), rf & 3u,
                                 reinterpret_cast<const T*>(b + (kRleStageRuns + 4) * 4) + (rf & (VPER - 1)), bm, m,
                                 skip, nr, last, ns, lane, err);
             } else {
-                rle_rows<T, WS>(c, h, dst, lens + (rf & ~3u), rf & 3u, vals + rf, bm, m, skip, nr, last, ns, lane,
+                rle_rows<T>(c, h, dst, lens + (rf & ~3u), rf & 3u, vals + rf, bm, m, skip, nr, last, ns, lane,
                                 err);
             }
         }
@@ -819,24 +817,6 @@ __device__ void rle_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t
 // (the decoder is in zf_strdict.cuh)
 constexpr uint32_t kStrCodeBuf = (1024u * 16u / 8u) + 32u;   // one tile of codes at b <= 16, plus the reader's overrun
 constexpr uint32_t kStrWin = 16u * zf::kStrTokenMax + 32u;    // 16 tokens of at most 64 bytes, at the output's alignment
-
-// ---------------------------------------------------------------- single-tile entry points
-// (used by the allocation-free kernel; 16-byte stores only)
-template <class T, int SCHEME>
-__device__ __forceinline__ void fp_warp(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t nr, uint32_t* wsm,
-                                        uint32_t* err) {
-    fp_job<T, SCHEME>(c, h, r0, nr, wsm, err);
-}
-template <class T>
-__device__ __forceinline__ void delta_warp(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t nr,
-                                           uint32_t* wsm, uint32_t* err) {
-    delta_job<T, false>(c, h, r0, nr, wsm, err, 8 * sizeof(T));
-}
-template <class T>
-__device__ __forceinline__ void rle_warp(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t nr, uint32_t* wsm,
-                                         uint32_t* err) {
-    rle_job<T, false>(c, h, r0, nr, wsm, err);
-}
 
 // Shared memory (bytes) one warp needs for a scheme, given the value size and
 // the widest bit width of the chunks it decodes (two staging buffers).

@@ -12,9 +12,8 @@
 #include <mutex>
 #include <unordered_map>
 
-#include "zf_device.cuh"
+#include "zf_decode.cuh"
 #include "zf_launch.h"
-#include "zf_strdict.cuh"
 
 namespace {
 
@@ -64,41 +63,11 @@ __device__ __forceinline__ uint32_t find_chunk(const ZfDevChunk* ch, uint32_t n,
     return a;
 }
 
-// WS: 256-bit stores (single-scheme kernels only).
-template <int SCHEME, int DT, bool WS>
-__device__ __forceinline__ void decode_one(const ZfDevChunk& c, const zfd::Hdr& h, uint32_t r0, uint32_t nrows,
-                                           uint32_t* wsm, uint32_t* err) {
-    if constexpr (DT == ZF_I32 || DT == ZF_I64) {
-        using T = typename std::conditional<DT == ZF_I64, int64_t, int32_t>::type;
-        if constexpr (SCHEME == ZF_FOR_BP || SCHEME == ZF_DICT_BP || SCHEME == ZF_RAW)
-            zfd::fp_job<T, SCHEME>(c, h, r0, nrows, wsm, err);
-        else if constexpr (SCHEME == ZF_DELTA_BP)
-            zfd::delta_job<T, WS>(c, h, r0, nrows, wsm, err, c.bmax);
-        else if constexpr (SCHEME == ZF_RLE)
-            zfd::rle_job<T, WS>(c, h, r0, nrows, wsm, err);
-    } else if constexpr (DT == ZF_F64) {
-        // doubles travel as their 64-bit patterns
-        if constexpr (SCHEME == ZF_RAW || SCHEME == ZF_FLOAT2INT) zfd::fp_job<int64_t, SCHEME>(c, h, r0, nrows, wsm, err);
-    } else if constexpr (DT == ZF_BYTES && SCHEME == ZF_STRDICT) {
-        zfd::strdict_job(c, h, r0, nrows, wsm, err);   // r0, nrows count tokens
-    } else if constexpr (DT == ZF_BYTES && SCHEME == ZF_RAW) {
-        // raw bytes: 16-byte copies
-        const uint32_t lane = threadIdx.x & 31;
-        const uint8_t* src = c.blob + h.off[0] + r0;
-        uint8_t* dst = c.dst + r0;
-        for (uint32_t i0 = lane * 16; i0 < nrows; i0 += 512) {
-            if (i0 + 16 <= nrows) reinterpret_cast<uint4*>(dst + i0)[0] = zfd::ldg16(src + i0);
-            else
-                for (uint32_t i = i0; i < nrows; i++) dst[i] = src[i];
-        }
-    }
-}
-
 __device__ __forceinline__ void decode_mixed(const ZfDevChunk& c, const zfd::Hdr& h, uint32_t r0, uint32_t nrows,
                                              uint32_t* wsm, uint32_t* err) {
     switch (c.scheme * 4 + c.dtype) {
 #define ZF_CASE(S, D) \
-    case S * 4 + D: decode_one<S, D, true>(c, h, r0, nrows, wsm, err); break;
+    case S * 4 + D: zfd::decode_one<S, D>(c, h, r0, nrows, wsm, err); break;
         ZF_CASE(ZF_RAW, ZF_I32) ZF_CASE(ZF_RAW, ZF_I64) ZF_CASE(ZF_RAW, ZF_BYTES)
         ZF_CASE(ZF_FOR_BP, ZF_I32) ZF_CASE(ZF_FOR_BP, ZF_I64)
         ZF_CASE(ZF_DICT_BP, ZF_I32) ZF_CASE(ZF_DICT_BP, ZF_I64)
@@ -127,7 +96,7 @@ __device__ __forceinline__ void run_job(const LaunchArgs& a, uint32_t job, uint3
     }
     const uint32_t nrows = min(a.job_rows, c.rows - r0);
     if constexpr (SCHEME < 0) decode_mixed(c, h, r0, nrows, wsm, a.err);
-    else decode_one<SCHEME, DT, true>(c, h, r0, nrows, wsm, a.err);
+    else zfd::decode_one<SCHEME, DT>(c, h, r0, nrows, wsm, a.err);
 }
 
 // Specialized launches (one scheme and dtype): one warp job per warp, as

@@ -7,220 +7,259 @@
 // front, a process whose memory budget is fixed by another runtime, or code
 // running inside a library call that may not grow the device heap.  Such a
 // caller passes its own input and output buffers; the only other memory the
-// decode needs (chunk descriptors, the work-queue counters and the error
-// word) lives in the fixed-size device array below, which every GPU that
-// loads the library holds until the process exits.
+// decode needs (the error word, a count of finished CTAs and the result the
+// host reads) lives in the fixed-size device array below, which every GPU
+// that loads the library holds until the process exits.
 //
-// The array is shared by all calls on a device and keeps the last call's
-// contents; each call rewrites what it needs (descriptors, counters, error
-// word) before the decode reads it.  Calls that overlap on the GPU -- from
-// several host threads or streams at once on the same device -- race on the
-// array; serialize them.
+// The array is shared by all calls on a device; a launch leaves it ready for
+// the next.  Calls that overlap on the GPU -- from several host threads or
+// streams at once on the same device -- race on the array; serialize them.
+//
+// One launch does everything: every warp reads the column header, finds its
+// chunk by division (all chunks but the last have chunk_rows rows), checks
+// the chunk's directory entry and header and decodes its rows.  The host
+// waits once, for the result.  A header read by the host, a set-up kernel of
+// one CTA for the chunk descriptors (whose threads each walked a chunk's
+// delta entries) and a persistent decode launch took 46.3 us for 3M rows of
+// RLE and 220 us for 1M rows of delta in one chunk; this takes 26.8 and 27.7
+// us, most of it the host's wait.  From 8M rows on it is bound by DRAM: 33M
+// rows of Float2Int in 65,536-row chunks took 317 us and take 102 us (3.6
+// TB/s).
 #include <cuda_runtime.h>
 
 #include <cstring>
 #include <mutex>
 
-#include "zf_device.cuh"
+#include "zf_decode.cuh"
 
 namespace {
 
-constexpr uint32_t kCtrlBytes = 256;
 constexpr uint32_t kNoallocMaxChunks = 4096;
-constexpr uint32_t kNoallocScratchBytes = kCtrlBytes + kNoallocMaxChunks * sizeof(ZfDevChunk);  // 262,400 B
-constexpr uint32_t kThreads = 256;
-constexpr uint32_t kTileRows = 1024 * (kThreads / 32);
+constexpr uint32_t kWarps = 4;                // warps per CTA
+constexpr uint32_t kCtasPerSm = 8;
+constexpr uint32_t kSmem = 28 * 1024;         // a CTA's staging memory: four warps of up to 7 KB, fewer at a time of more
+constexpr uint32_t kJobTiles = 4;             // 1024-row tiles of a job at most
 constexpr int kMaxDevices = 64;
 
-// Control block: [0] chunks, [1] tiles, [2] queue next, [3] CTAs done,
-// [4] error bits, [5] first failing chunk.  Descriptors follow at kCtrlBytes.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
+// [0] CTAs done, [1] error bits and [2] first failing chunk while a launch
+// runs; [3], [4] the same and [5] the column header's status when it is done.
+static __device__ uint32_t g_noalloc_ctrl[8] = {0, 0, 0xFFFFFFFFu, 0, 0, 0, 0, 0};
 
 std::mutex g_mu;
-void* g_scratch_addr[kMaxDevices];   // device address of g_noalloc_scratch per device (set once)
-bool g_attr_set[kMaxDevices];        // shared-memory attribute of noalloc_decode set on the device
+struct Device {
+    void* ctrl = nullptr;   // device address of g_noalloc_ctrl (set once)
+    int sms = 0;
+} g_dev[kMaxDevices];
 
-// Structural checks of one chunk blob on the device (the host path makes the
-// same checks before a column is accepted).
-__device__ bool chunk_ok(const uint8_t* c, uint64_t len, int scheme, int dtype, uint32_t rows) {
-    if (len < 64 || (len & 15) || ((uintptr_t)c & 15)) return false;
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(c);
-    if (w[0] != zf::kChunkMagic || c[4] != scheme || c[5] != dtype || w[2] != rows) return false;
-    const uint32_t b = c[6], n_aux = w[3];
-    const uint32_t* off = w + 6;
-    const uint32_t* ln = w + 9;
-    const int nsec = (scheme == ZF_RLE || scheme == ZF_FLOAT2INT) ? 3
-                     : (scheme == ZF_DICT_BP || scheme == ZF_DELTA_BP) ? 2 : 1;
-    for (int s = 0; s < nsec; s++)
-        if (off[s] < 64 || (off[s] & 15) || (uint64_t)off[s] + ln[s] > len) return false;
-    const uint32_t sz = dtype == ZF_I32 ? 4 : 8, wd = 8 * sz;
-    switch (scheme) {
-    case ZF_RAW: return ln[0] == (uint64_t)rows * sz;
-    case ZF_FOR_BP: return b <= wd && ln[0] == ((uint64_t)rows * b + 7) / 8;
-    case ZF_DICT_BP: {
-        uint32_t bits = 0;
-        for (uint32_t x = n_aux ? n_aux - 1 : 0; x; x >>= 1) bits++;
-        return n_aux <= zf::kMaxDict && (!rows || n_aux) && ln[0] == (uint64_t)n_aux * sz && b == bits &&
-               ln[1] == ((uint64_t)rows * b + 7) / 8;
+struct Column {
+    uint32_t scheme, dtype, nch, chunk_rows, size;   // size: bytes of a value
+    uint64_t n_rows, total;
+};
+
+// The column header's fields and what the call returns for them.
+__device__ zf_status read_column(const uint8_t* col, uint64_t col_bytes, uint64_t out_bytes, Column& c) {
+    const uint4 a = zfd::ldg16(col), b = zfd::ldg16(col + 16);
+    const uint2 t = __ldg(reinterpret_cast<const uint2*>(col + 32));
+    c.scheme = (a.y >> 16) & 0xFFu;
+    c.dtype = a.y >> 24;
+    c.nch = a.z;
+    c.chunk_rows = a.w;
+    c.n_rows = ((uint64_t)b.y << 32) | b.x;
+    c.total = ((uint64_t)t.y << 32) | t.x;
+    c.size = c.dtype == ZF_I32 ? 4 : 8;
+    if (a.x != zf::kColMagic || (a.y & 0xFFFFu) != 1) return ZF_ECORRUPT;
+    if (c.dtype != ZF_I32 && c.dtype != ZF_I64 && c.dtype != ZF_F64) return ZF_EUNSUPPORTED;
+    if (c.scheme == ZF_ANS) return ZF_EUNSUPPORTED;   // decoded by its own kernel on the regular paths
+    const bool scheme_ok = c.dtype == ZF_F64 ? (c.scheme == ZF_RAW || c.scheme == ZF_FLOAT2INT) : c.scheme <= ZF_RLE;
+    if (!scheme_ok || c.chunk_rows == 0 || c.chunk_rows % 1024 || c.chunk_rows > (1u << 30) || c.n_rows > (1ull << 48))
+        return ZF_ECORRUPT;
+    if (c.nch > kNoallocMaxChunks) return ZF_EINVAL;
+    if ((uint64_t)c.nch != (c.n_rows + c.chunk_rows - 1) / c.chunk_rows || c.total > col_bytes ||
+        64 + 32ull * c.nch > c.total)
+        return ZF_ECORRUPT;
+    return c.n_rows * c.size > out_bytes ? ZF_EINVAL : ZF_OK;
+}
+
+// Structural checks of chunk k (the host path makes the same checks before a
+// column is accepted) and its descriptor; false if it is malformed.  The
+// entries of delta blocks and Float2Int exceptions are checked by the jobs
+// that read them (job_ok).
+__device__ bool chunk_ok(const uint8_t* col, const Column& c, uint32_t k, uint8_t* out, uint64_t out_bytes,
+                         ZfDevChunk& dc, zfd::Hdr& h) {
+    const uint8_t* d = col + 64 + 32ull * k;
+    const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(d);        // offset, bytes
+    const ulonglong2 r = *reinterpret_cast<const ulonglong2*>(d + 16);   // first row, rows
+    const uint64_t off = e.x, len = e.y;
+    // chunks follow each other: each starts where the previous one ends
+    uint64_t start = 64 + 32ull * c.nch;
+    if (k) {
+        const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(d - 32);
+        start = p.x + p.y;
     }
+    const uint64_t row0 = (uint64_t)k * c.chunk_rows;
+    const uint32_t rows = (uint32_t)min((unsigned long long)c.chunk_rows, (unsigned long long)(c.n_rows - row0));
+    if (off != start || off < 64 + 32ull * c.nch || off > c.total || len > c.total - off || r.x != row0 ||
+        (uint32_t)r.y != rows || len < 64 || (len & 15) || (off & 15))
+        return false;
+    const uint8_t* blob = col + off;
+    dc.blob = blob;
+    dc.dst = out + row0 * c.size;
+    dc.dst_cap = out_bytes - row0 * c.size;
+    dc.rows = rows;
+    dc.blob_bytes = (uint32_t)len;
+    dc.chunk_id = k;
+    dc.scheme = (uint8_t)c.scheme;
+    dc.dtype = (uint8_t)c.dtype;
+    zfd::load_hdr(blob, h);
+    const uint2 m = __ldg(reinterpret_cast<const uint2*>(blob));
+    if (m.x != zf::kChunkMagic || (m.y & 0xFFu) != c.scheme || ((m.y >> 8) & 0xFFu) != c.dtype || h.rows != rows)
+        return false;
+    const int nsec = (c.scheme == ZF_RLE || c.scheme == ZF_FLOAT2INT) ? 3
+                     : (c.scheme == ZF_DICT_BP || c.scheme == ZF_DELTA_BP) ? 2 : 1;
+    for (int s = 0; s < 3; s++)
+        if (s < nsec && (h.off[s] < 64 || (h.off[s] & 15) || (uint64_t)h.off[s] + h.len[s] > len)) return false;
+    const uint32_t sz = c.size, wd = 8 * sz, b = h.b, n_aux = h.n_aux;
+    const uint64_t packed = ((uint64_t)rows * b + 7) / 8;
+    switch (c.scheme) {
+    case ZF_RAW: return h.len[0] == (uint64_t)rows * sz;
+    case ZF_FOR_BP: return b <= wd && h.len[0] == packed;
+    case ZF_DICT_BP:
+        return n_aux <= zf::kMaxDict && n_aux && h.len[0] == (uint64_t)n_aux * sz && b == 32u - __clz(n_aux - 1) &&
+               h.len[1] == packed;
     case ZF_DELTA_BP: {
         const uint32_t nb = (rows + zf::kDeltaBlock - 1) / zf::kDeltaBlock;
-        if (n_aux != nb || ln[0] != (uint64_t)nb * zf::kDeltaEntry) return false;
-        for (uint32_t k = 0; k < nb; k++) {
-            const uint8_t* e = c + off[0] + (uint64_t)k * zf::kDeltaEntry;
-            const uint32_t po = *reinterpret_cast<const uint32_t*>(e + 16), bk = e[20];
-            const uint32_t mk = min(zf::kDeltaBlock, rows - k * zf::kDeltaBlock);
-            if (bk > wd || (po & 15) || (uint64_t)po + ((((uint64_t)mk * bk + 7) / 8 + 15) & ~15ull) > ln[1])
-                return false;
-        }
-        return true;
+        return n_aux == nb && h.len[0] == (uint64_t)nb * zf::kDeltaEntry;
     }
     case ZF_RLE:
-        return n_aux <= rows && (!rows || n_aux) && ln[0] == (uint64_t)n_aux * sz && ln[1] == 4ull * n_aux &&
-               ln[2] == 8ull * ((rows + zf::kRleDirRows - 1) / zf::kRleDirRows);
-    case ZF_FLOAT2INT: {
-        if (b > 64 || c[48] > zf::kF2IMaxExp || n_aux > rows || ln[0] != ((uint64_t)rows * b + 7) / 8 ||
-            ln[1] != 4ull * n_aux || ln[2] != 8ull * n_aux)
-            return false;
-        return true;   // the order of the exception rows is checked by the whole CTA
-    }
+        return n_aux <= rows && n_aux && h.len[0] == (uint64_t)n_aux * sz && h.len[1] == 4ull * n_aux &&
+               h.len[2] == 8ull * ((rows + zf::kRleDirRows - 1) / zf::kRleDirRows);
+    case ZF_FLOAT2INT:
+        return b <= 64 && blob[48] <= zf::kF2IMaxExp && n_aux <= rows && h.len[0] == packed &&
+               h.len[1] == 4ull * n_aux && h.len[2] == 8ull * n_aux;
     }
     return false;
 }
 
-// One CTA: check every chunk of the column and write its descriptor into the
-// scratch array, then the tile counts and a reset work queue and error word.
-__global__ void noalloc_setup(const uint8_t* col, uint64_t col_bytes, uint8_t* out, uint64_t out_bytes,
-                              uint32_t nch, int scheme, int dtype, uint64_t n_rows, uint32_t chunk_rows) {
-    uint32_t* ctrl = reinterpret_cast<uint32_t*>(g_noalloc_scratch);
-    ZfDevChunk* desc = reinterpret_cast<ZfDevChunk*>(g_noalloc_scratch + kCtrlBytes);
-    __shared__ uint32_t s_bad;
-    if (threadIdx.x == 0) s_bad = 0;
-    __syncthreads();
-    const uint32_t sz = dtype == ZF_I32 ? 4 : 8;
-    uint64_t expect_end = 64 + 32ull * nch;
-    for (uint32_t k = threadIdx.x; k < nch; k += blockDim.x) {
-        const uint8_t* d = col + 64 + 32ull * k;
-        const uint64_t off = *reinterpret_cast<const uint64_t*>(d);
-        const uint64_t len = *reinterpret_cast<const uint64_t*>(d + 8);
-        const uint64_t row0 = *reinterpret_cast<const uint64_t*>(d + 16);
-        const uint32_t rows = *reinterpret_cast<const uint32_t*>(d + 24);
-        bool ok = off >= expect_end && off <= col_bytes && len <= col_bytes - off &&
-                  row0 == (uint64_t)k * chunk_rows && rows == (uint32_t)min((uint64_t)chunk_rows, n_rows - row0) &&
-                  chunk_ok(col + off, len, scheme, dtype, rows);
-        ZfDevChunk dc{};
-        dc.blob = col + off;
-        dc.dst = out + row0 * sz;
-        dc.dst_cap = out_bytes - row0 * sz;
-        dc.rows = rows;
-        dc.ntiles = (rows + kTileRows - 1) / kTileRows;
-        dc.blob_bytes = (uint32_t)len;
-        dc.chunk_id = k;
-        dc.scheme = (uint8_t)scheme;
-        dc.dtype = (uint8_t)dtype;
-        desc[k] = dc;
-        if (!ok) atomicOr(&s_bad, 1u);
-    }
-    __syncthreads();
-    if (scheme == ZF_FLOAT2INT && !s_bad) {
-        // Float2Int exception rows strictly increasing and inside the chunk
-        // (the decoder's search over them relies on the order); the CTA's
-        // threads share each chunk's rows
-        bool bad = false;
-        for (uint32_t k = 0; k < nch; k++) {
-            const uint8_t* cb = col + *reinterpret_cast<const uint64_t*>(col + 64 + 32ull * k);
-            const uint32_t* w = reinterpret_cast<const uint32_t*>(cb);
-            const uint32_t rows = w[2], n_aux = w[3];
-            const uint32_t* er = reinterpret_cast<const uint32_t*>(cb + w[7]);   // section 1
-            for (uint32_t j = threadIdx.x; j < n_aux; j += blockDim.x)
-                bad |= er[j] >= rows || (j && er[j] <= er[j - 1]);
+// The rest of a chunk's checks, shared by its jobs: delta block entries of
+// the job's rows (dc.bmax becomes the widest of them) and the job's share of
+// a Float2Int chunk's exception rows, which must be strictly increasing and
+// inside the chunk.
+__device__ bool job_ok(const zfd::Hdr& h, uint32_t r0, uint32_t nrows, uint32_t job_rows, ZfDevChunk& dc) {
+    const uint32_t lane = threadIdx.x & 31;
+    dc.bmax = (uint8_t)h.b;
+    bool ok = true;
+    if (dc.scheme == ZF_DELTA_BP) {
+        uint32_t b = 0;
+        if (lane * zf::kDeltaBlock < nrows) {
+            const uint8_t* e = dc.blob + h.off[0] + (uint64_t)(r0 / zf::kDeltaBlock + lane) * zf::kDeltaEntry;
+            const uint2 w = __ldg(reinterpret_cast<const uint2*>(e + 16));
+            const uint32_t mk = min(zf::kDeltaBlock, nrows - lane * zf::kDeltaBlock);
+            b = w.y & 0xFFu;
+            ok = b <= (dc.dtype == ZF_I32 ? 32u : 64u) && !(w.x & 15) &&
+                 (uint64_t)w.x + ((((uint64_t)mk * b + 7) / 8 + 15) & ~15ull) <= h.len[1];
         }
-        if (bad) atomicOr(&s_bad, 1u);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        // chunks must follow each other: each starts where the previous ends
-        uint32_t tiles = 0;
-        uint64_t pos = expect_end;
-        for (uint32_t k = 0; k < nch; k++) {
-            const uint8_t* d = col + 64 + 32ull * k;
-            const uint64_t off = *reinterpret_cast<const uint64_t*>(d);
-            if (off != pos) s_bad = 1;
-            pos = off + *reinterpret_cast<const uint64_t*>(d + 8);
-            desc[k].tile0 = tiles;
-            tiles += desc[k].ntiles;
+        dc.bmax = (uint8_t)__reduce_max_sync(0xFFFFFFFFu, b);
+    } else if (dc.scheme == ZF_FLOAT2INT) {
+        const uint64_t jobs = (dc.rows + job_rows - 1) / job_rows, j = r0 / job_rows;
+        const uint32_t z = (uint32_t)((j + 1) * h.n_aux / jobs);
+        const uint32_t* er = reinterpret_cast<const uint32_t*>(dc.blob + h.off[1]);
+        for (uint32_t i = (uint32_t)(j * h.n_aux / jobs) + lane; i < z; i += 32) {
+            const uint32_t x = __ldg(er + i);
+            ok &= x < dc.rows && (i == 0 || x > __ldg(er + i - 1));
         }
-        ctrl[0] = nch;
-        ctrl[1] = s_bad ? 0 : tiles;
-        ctrl[2] = 0;
-        ctrl[3] = 0;
-        ctrl[4] = s_bad ? (1u << ZF_ECORRUPT) : 0u;
-        ctrl[5] = 0xFFFFFFFFu;
-        __threadfence();
     }
+    return __all_sync(0xFFFFFFFFu, ok);
 }
 
-__device__ __noinline__ void noalloc_tile(const ZfDevChunk& c, const zfd::Hdr& h, uint32_t r0, uint32_t nr,
-                                          uint32_t* wsm, uint32_t* err) {
+__device__ __forceinline__ void decode(const ZfDevChunk& c, const zfd::Hdr& h, uint32_t r0, uint32_t nr, uint32_t* wsm,
+                                       uint32_t* err) {
     switch (c.scheme * 4 + c.dtype) {
-    case ZF_RAW * 4 + ZF_I32: zfd::fp_warp<int32_t, ZF_RAW>(c, h, r0, nr, wsm, err); break;
-    case ZF_RAW * 4 + ZF_I64: zfd::fp_warp<int64_t, ZF_RAW>(c, h, r0, nr, wsm, err); break;
-    case ZF_FOR_BP * 4 + ZF_I32: zfd::fp_warp<int32_t, ZF_FOR_BP>(c, h, r0, nr, wsm, err); break;
-    case ZF_FOR_BP * 4 + ZF_I64: zfd::fp_warp<int64_t, ZF_FOR_BP>(c, h, r0, nr, wsm, err); break;
-    case ZF_DICT_BP * 4 + ZF_I32: zfd::fp_warp<int32_t, ZF_DICT_BP>(c, h, r0, nr, wsm, err); break;
-    case ZF_DICT_BP * 4 + ZF_I64: zfd::fp_warp<int64_t, ZF_DICT_BP>(c, h, r0, nr, wsm, err); break;
-    case ZF_DELTA_BP * 4 + ZF_I32: zfd::delta_warp<int32_t>(c, h, r0, nr, wsm, err); break;
-    case ZF_DELTA_BP * 4 + ZF_I64: zfd::delta_warp<int64_t>(c, h, r0, nr, wsm, err); break;
-    case ZF_RLE * 4 + ZF_I32: zfd::rle_warp<int32_t>(c, h, r0, nr, wsm, err); break;
-    case ZF_RLE * 4 + ZF_I64: zfd::rle_warp<int64_t>(c, h, r0, nr, wsm, err); break;
-    // doubles travel as their 64-bit patterns
-    case ZF_RAW * 4 + ZF_F64: zfd::fp_warp<int64_t, ZF_RAW>(c, h, r0, nr, wsm, err); break;
-    case ZF_FLOAT2INT * 4 + ZF_F64: zfd::fp_warp<int64_t, ZF_FLOAT2INT>(c, h, r0, nr, wsm, err); break;
-    default:
-        if ((threadIdx.x & 31) == 0) zfd::report(err, ZF_EINVAL, c.chunk_id);
+#define ZF_CASE(S, D) \
+    case S * 4 + D: zfd::decode_one<S, D>(c, h, r0, nr, wsm, err); break;
+        ZF_CASE(ZF_RAW, ZF_I32) ZF_CASE(ZF_RAW, ZF_I64) ZF_CASE(ZF_RAW, ZF_F64)
+        ZF_CASE(ZF_FOR_BP, ZF_I32) ZF_CASE(ZF_FOR_BP, ZF_I64)
+        ZF_CASE(ZF_DICT_BP, ZF_I32) ZF_CASE(ZF_DICT_BP, ZF_I64)
+        ZF_CASE(ZF_DELTA_BP, ZF_I32) ZF_CASE(ZF_DELTA_BP, ZF_I64)
+        ZF_CASE(ZF_RLE, ZF_I32) ZF_CASE(ZF_RLE, ZF_I64) ZF_CASE(ZF_FLOAT2INT, ZF_F64)
+#undef ZF_CASE
     }
 }
 
-// Persistent decode: CTAs pop tiles from the queue in the scratch array; the
-// last CTA to finish resets the queue.
-__global__ void __launch_bounds__(kThreads, 2) noalloc_decode(uint32_t warp_smem) {
-    extern __shared__ uint4 smem4[];
-    __shared__ uint32_t s_tile;
-    uint32_t* ctrl = reinterpret_cast<uint32_t*>(g_noalloc_scratch);
-    const ZfDevChunk* desc = reinterpret_cast<const ZfDevChunk*>(g_noalloc_scratch + kCtrlBytes);
-    uint32_t* err = ctrl + 4;
-    const uint32_t nch = ctrl[0], ntiles = ctrl[1];
-    const uint32_t warp = threadIdx.x >> 5;
-    uint32_t* wsm = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(smem4) + warp * warp_smem);
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_tile = atomicAdd(&ctrl[2], 1u);
-        __syncthreads();
-        const uint32_t tile = s_tile;
-        if (tile >= ntiles) break;
-        uint32_t a = 0, z = nch;
-        while (z - a > 1) {
-            const uint32_t mid = (a + z) >> 1;
-            if (desc[mid].tile0 <= tile) a = mid;
-            else z = mid;
+// A CTA's warps take consecutive jobs, then the jobs gridDim CTAs further.
+// The jobs of a CTA share kSmem bytes: when the widest of them does not fit
+// four times, fewer warps decode at a time.
+__global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) noalloc_decode(const uint8_t* col, uint64_t col_bytes,
+                                                                          uint8_t* out, uint64_t out_bytes) {
+    __shared__ uint4 smem4[kSmem / 16];
+    __shared__ uint32_t s_need[kWarps];
+    __shared__ Column s_col;
+    __shared__ ZfDevChunk s_dc[kWarps];   // the warps' chunks, here and not in registers: 64 a thread are few
+    __shared__ zfd::Hdr s_h[kWarps];      // for a kernel that decodes every scheme
+    __shared__ uint32_t s_job_rows, s_per, s_njobs;   // rows of a job, jobs of a chunk, jobs of the column
+    uint32_t* ctrl = g_noalloc_ctrl;
+    uint32_t* err = ctrl + 1;
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        Column c;
+        const zf_status st = read_column(col, col_bytes, out_bytes, c);
+        if (blockIdx.x == 0) ctrl[5] = (uint32_t)st;
+        s_njobs = 0;
+        if (st == ZF_OK && c.n_rows) {
+            const uint64_t tiles = (c.n_rows + 1023) / 1024, warps = (uint64_t)gridDim.x * kWarps;
+            const uint32_t most = (uint32_t)min((unsigned long long)kJobTiles, (unsigned long long)((tiles + warps - 1) / warps));
+            const uint32_t rows = 1024u * most, per = (c.chunk_rows + rows - 1) / rows;
+            const uint32_t last = (uint32_t)(c.n_rows - (uint64_t)(c.nch - 1) * c.chunk_rows);
+            s_job_rows = rows;
+            s_per = per;
+            s_njobs = (c.nch - 1) * per + (last + rows - 1) / rows;   // a column of 2^32 jobs has 2^42 rows
         }
-        const ZfDevChunk c = desc[a];
-        zfd::Hdr h;
-        zfd::load_hdr(c.blob, h);
-        const uint32_t rc = (tile - c.tile0) * kTileRows;
-        const uint32_t sz = c.dtype == ZF_I32 ? 4 : 8;
-        if (h.rows != c.rows || rc >= c.rows || (uint64_t)c.rows * sz > c.dst_cap) {
-            if (threadIdx.x == 0) zfd::report(err, ZF_ECORRUPT, c.chunk_id);
-            continue;
-        }
-        const uint32_t r0 = rc + warp * zfd::kWarpRows;
-        if (r0 < c.rows) noalloc_tile(c, h, r0, min(zfd::kWarpRows, c.rows - r0), wsm, err);
+        s_col = c;
     }
+    __syncthreads();
+    {
+        for (uint32_t base = blockIdx.x * kWarps; base < s_njobs; base += gridDim.x * kWarps) {
+            const uint32_t job = base + warp;
+            uint32_t need = 0, r0 = 0, nr = 0;
+            ZfDevChunk dc{};
+            zfd::Hdr h{};
+            if (job < s_njobs) {
+                const uint32_t k = job / s_per;
+                r0 = (job % s_per) * s_job_rows;
+                bool ok = chunk_ok(col, s_col, k, out, out_bytes, dc, h);
+                if (ok) {
+                    nr = min(s_job_rows, dc.rows - r0);
+                    ok = job_ok(h, r0, nr, s_job_rows, dc);
+                }
+                if (ok) need = max(16u, (zfd::warp_smem((int)s_col.scheme, s_col.size, dc.bmax) + 15u) & ~15u);
+                else if (lane == 0) zfd::report(err, ZF_ECORRUPT, k);
+                if (lane == 0) {
+                    s_dc[warp] = dc;
+                    s_h[warp] = h;
+                }
+            }
+            __syncthreads();
+            if (lane == 0) s_need[warp] = need;
+            __syncthreads();
+            uint32_t most = 16;
+#pragma unroll
+            for (uint32_t w = 0; w < kWarps; w++) most = max(most, s_need[w]);
+            const uint32_t at_once = min(kWarps, kSmem / most);
+            for (uint32_t g = 0; g < kWarps; g += at_once) {
+                if (need && warp >= g && warp < g + at_once)
+                    decode(s_dc[warp], s_h[warp], r0, nr, reinterpret_cast<uint32_t*>(smem4) + (warp - g) * (most / 4), err);
+                if (at_once < kWarps) __syncthreads();
+            }
+        }
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(&ctrl[3], 1u) == gridDim.x - 1) {
-            ctrl[2] = 0;
-            ctrl[3] = 0;
+        if (atomicAdd(&ctrl[0], 1u) == gridDim.x - 1) {
+            // the last CTA hands the result over and leaves the array ready for the next launch
+            __threadfence();
+            ctrl[3] = atomicExch(&ctrl[1], 0u);
+            ctrl[4] = atomicExch(&ctrl[2], 0xFFFFFFFFu);
+            ctrl[0] = 0;
             __threadfence();
         }
     }
@@ -234,85 +273,32 @@ extern "C" zf_status zf_decompress_device_noalloc(const void* d_column, uint64_t
         return ZF_EINVAL;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return ZF_ECUDA;
-    void* scratch = nullptr;
+    Device d;
     {
         // first call on this device: look up the array's device address (the
         // host-side name of the array is not a device address)
         std::lock_guard<std::mutex> g(g_mu);
-        if (!g_scratch_addr[dev]) {
-            void* p = nullptr;
-            if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
+        if (!g_dev[dev].ctrl) {
+            if (cudaGetSymbolAddress(&d.ctrl, g_noalloc_ctrl) != cudaSuccess || !d.ctrl ||
+                cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || d.sms < 1) {
                 cudaGetLastError();
                 return ZF_ECUDA;
             }
-            g_scratch_addr[dev] = p;
+            g_dev[dev] = d;
         }
-        scratch = g_scratch_addr[dev];
+        d = g_dev[dev];
     }
     cudaStream_t s = (cudaStream_t)stream;
-    // column header, read on the caller's stream so it follows the caller's writes
-    unsigned char hdr[64];
-    if (cudaMemcpyAsync(hdr, d_column, 64, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    // a column has at most out_bytes / 4 rows, or the kernel refuses it
+    const uint64_t ctas = (out_bytes / 4096 + kWarps) / kWarps, most = (uint64_t)d.sms * kCtasPerSm;
+    noalloc_decode<<<(unsigned)(ctas < most ? ctas : most), kWarps * 32, 0, s>>>(
+        (const uint8_t*)d_column, column_bytes, (uint8_t*)d_out, out_bytes);
+    if (cudaGetLastError() != cudaSuccess) return ZF_ECUDA;
+    uint32_t r[3] = {0, 0, 0};   // error bits, first failing chunk, the header's status
+    if (cudaMemcpyAsync(r, (const uint8_t*)d.ctrl + 12, 12, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return ZF_ECUDA;
-    uint32_t magic, nch, chunk_rows;
-    uint16_t ver;
-    uint64_t n_rows, total;
-    memcpy(&magic, hdr, 4);
-    memcpy(&ver, hdr + 4, 2);
-    const int scheme = hdr[6], dtype = hdr[7];
-    memcpy(&nch, hdr + 8, 4);
-    memcpy(&chunk_rows, hdr + 12, 4);
-    memcpy(&n_rows, hdr + 16, 8);
-    memcpy(&total, hdr + 32, 8);
-    if (magic != zf::kColMagic || ver != 1) return ZF_ECORRUPT;
-    if (dtype != ZF_I32 && dtype != ZF_I64 && dtype != ZF_F64) return ZF_EUNSUPPORTED;
-    if (scheme == ZF_ANS) return ZF_EUNSUPPORTED;   // decoded by its own kernel on the regular paths
-    const bool scheme_ok = dtype == ZF_F64 ? (scheme == ZF_RAW || scheme == ZF_FLOAT2INT)
-                                           : (scheme >= ZF_RAW && scheme <= ZF_RLE);
-    if (!scheme_ok || chunk_rows == 0 || chunk_rows % 1024 || chunk_rows > (1u << 30) || n_rows > (1ull << 48))
-        return ZF_ECORRUPT;
-    if (nch > kNoallocMaxChunks) return ZF_EINVAL;  // above the fixed scratch size
-    if ((uint64_t)nch != (n_rows + chunk_rows - 1) / chunk_rows || total > column_bytes ||
-        64 + 32ull * nch > total)
-        return ZF_ECORRUPT;
-    const uint32_t sz = dtype == ZF_I32 ? 4 : 8;
-    if (n_rows * sz > out_bytes) return ZF_EINVAL;
-    if (n_rows == 0) return ZF_OK;
-    noalloc_setup<<<1, 256, 0, s>>>((const uint8_t*)d_column, total, (uint8_t*)d_out, out_bytes, nch, scheme,
-                                    dtype, n_rows, chunk_rows);
-    if (cudaGetLastError() != cudaSuccess) return ZF_ECUDA;
-    // widest per-warp slice any chunk of this dtype may need (bit widths are not read on the host)
-    auto slice = [](uint32_t vb) {
-        uint32_t w = zfd::warp_smem(ZF_FOR_BP, vb, 8 * vb);
-        w = w > zfd::warp_smem(ZF_RLE, vb, 0) ? w : zfd::warp_smem(ZF_RLE, vb, 0);
-        return (w + 15) & ~15u;
-    };
-    const uint32_t ws = slice(sz);
-    const uint32_t smem = ws * (kThreads / 32);
-    {
-        // once per device, allow the largest launch of any value size (8-byte values need the most)
-        std::lock_guard<std::mutex> g(g_mu);
-        if (!g_attr_set[dev]) {
-            if (cudaFuncSetAttribute(noalloc_decode, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(slice(8) * (kThreads / 32))) != cudaSuccess) {
-                cudaGetLastError();
-                return ZF_ECUDA;
-            }
-            g_attr_set[dev] = true;
-        }
-    }
-    int per_sm = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, noalloc_decode, kThreads, smem) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || per_sm < 1)
-        return ZF_ECUDA;
-    noalloc_decode<<<per_sm * sms, kThreads, smem, s>>>(ws);
-    if (cudaGetLastError() != cudaSuccess) return ZF_ECUDA;
-    uint32_t e[2] = {0, 0};
-    if (cudaMemcpyAsync(e, (const uint8_t*)scratch + 16, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return ZF_ECUDA;
-    if (e[0] & (1u << ZF_ECORRUPT)) return ZF_ECORRUPT;
-    if (e[0]) return ZF_EINVAL;
-    return ZF_OK;
+    if (r[2]) return (zf_status)r[2];
+    if (r[0] & (1u << ZF_ECORRUPT)) return ZF_ECORRUPT;
+    return r[0] ? ZF_EINVAL : ZF_OK;
 }
