@@ -17,131 +17,156 @@ namespace {
 
 constexpr uint32_t kWarps = zf::kAnsJobsPerCta;   // warps (jobs) per CTA, all of one chunk
 
-// The CTA's tables for its chunk.  Slot entry: symbol << 24 | (slot - c) <<
-// 12 | (f - 1), so a decode step finds the symbol, its frequency f and the
-// slot's offset in the symbol's range [c, c + f) with one shared load.
+constexpr uint32_t kRing = 4;                     // 16-byte words of a lane's stream in shared memory
+
+// The CTA's tables for its chunk.  A slot's entry holds its symbol, the
+// symbol's frequency f and the slot's offset in the symbol's range [c, c + f),
+// so a decode step takes one shared load for the state and one for the value.
+// Up to 128 symbols: f << 19 | symbol << 12 | (slot - c), where a shift gives
+// f; more (WIDE): symbol << 24 | (f - 1) << 12 | (slot - c).
 struct AnsSmem {
     uint32_t slot[zf::kAnsM];
     unsigned long long val[zf::kAnsMaxSymbols];   // the symbols' values (64-bit patterns)
     uint32_t cum[zf::kAnsMaxSymbols + 1];         // cumulative frequencies, cum[nd] = M
     uint32_t wsum[kWarps];
+    uint4 ring[kWarps * 32][kRing + 1];           // per lane: 16-byte word c of s2 at c mod kRing (one more: spreads the banks)
 };
 
+template <bool WIDE>
+__device__ __forceinline__ uint32_t ans_entry(uint32_t sym, uint32_t f, uint32_t d) {
+    return WIDE ? (sym << 24) | ((f - 1u) << 12) | d : (f << 19) | (sym << 12) | d;
+}
+
 // Stream k of the chunk, rows [k L, k L + n), decoded by one lane.  The
-// stream's bytes [a0, a1) of s2 come through a 64-bit buffer, next byte in
-// the top bits.  Per row: the slot entry of x mod M gives the value and
-// x = f (x >> 12) + (slot - c); then zero, one or two bytes enter while
-// x < L (after a step x >= 2^11): one funnel shift of x over the buffer's
-// top word, and the buffer moves up by as many bytes.  A row takes at most
-// two bytes, so the buffer is topped up to 64 bits before every four rows,
-// by every lane at once (no lane waits on another's refill): two aligned
-// 8-byte loads from the word holding the next byte (words past the stream's
-// last one read as zero; s2 starts on a 16-byte boundary of the blob, so a
-// word holding a stream byte lies inside the blob).  Bytes past the stream
-// may enter the buffer; a valid stream never takes them.
+// stream's bytes [a0, a1) of s2 pass through a window of two 32-bit words,
+// first byte on top.  Per row: the slot entry of x mod M gives the value and
+// x = f (x >> 12) + (slot - c); then zero, one or two bytes enter while x < L
+// (after a step x >= 2^11): one shift of the window brings its next 16 bits to
+// the top, a funnel shift moves them into x.  A row takes at most two bytes, so
+// the window moves up by a word after every second row at the most, by every
+// lane at once (no lane waits on another's refill).  The words come from a
+// ring of 64 bytes per lane that cp.async keeps ahead: eight rows take at most
+// 16 bytes and the window reaches 15 further, so before every eight rows the
+// third 16-byte word from the current one is asked for and the one asked for
+// eight rows earlier is there.  (A refill from global memory holds up the
+// whole warp: 93 us for 0.3M rows, where this takes 46.)  Only words that
+// hold stream bytes are asked for (s2 starts on a 16-byte boundary of the blob,
+// so they lie inside it); what the ring holds past the stream may enter the
+// window, a valid stream never takes it.
 // Eight int32 or four int64 rows leave as one 32-byte sector.  Returns true
 // if the stream is malformed: it must use exactly its bytes and end at x = L.
-// SMALL (a chunk of at most four values): the symbol of a slot is found by
-// comparing it with the cumulative frequencies, held in registers with the
-// frequencies and values, so a row's dependent chain has no shared-memory
-// lookup (whose address is the previous row's state).
-template <class T, bool SMALL>
-__device__ __forceinline__ bool ans_stream(const AnsSmem& sm, const uint8_t* s2, uint32_t a0, uint32_t a1, T* dst,
+// What bounds it: the latency of a row's dependent chain (slot lookup among
+// bank conflicts, multiply-add, renormalization), with the 27 warps per SM that
+// the streams of 64M rows give and more so with fewer; about 30 instructions a
+// row.  Symbols of up to four values found by compares in registers, with a
+// 64-bit byte buffer topped up every four rows, took 41 instructions and
+// bound the ALU pipe; larger alphabets took a lookup and the same buffer.
+// Resident calls of 64M int32 rows in 512-row streams, before and now: 3
+// values 157 and 108 us (2.6 TB/s), 16 values 206 and 114, 200 values 231 and
+// 137; 4M rows of 3 values 61 and 46.  A window refilled without a branch (the
+// ring is then read by every lane) added 5 us.
+template <class T, bool WIDE>
+__device__ __forceinline__ bool ans_stream(AnsSmem& sm, const uint8_t* s2, uint32_t a0, uint32_t a1, T* dst,
                                            uint32_t n) {
-    const unsigned long long* w8 = reinterpret_cast<const unsigned long long*>(s2);
-    const uint32_t lastw = (a1 - 1) >> 3;   // the last word holding a stream byte (a1 > a0)
-    uint32_t pos = a0;                      // next stream byte to enter the buffer
-    unsigned long long bb = 0;              // buffered bytes, the next one in bits 63..56
-    uint32_t nbits = 0;                     // buffered bits, a multiple of 8 in [0, 64]
-    auto topup = [&]() {
-        const uint32_t need = (64u - nbits) >> 3;
-        const uint32_t wi = pos >> 3, s = 8u * (pos & 7u);
-        const unsigned long long w0 = wi <= lastw ? __ldg(w8 + wi) : 0ull;
-        const unsigned long long w1 = wi + 1 <= lastw ? __ldg(w8 + wi + 1) : 0ull;
-        // the 8 bytes from pos, little-endian: (w1:w0) >> s
-        const bool lo = s < 32;
-        const uint32_t q0 = lo ? (uint32_t)w0 : (uint32_t)(w0 >> 32), q1 = lo ? (uint32_t)(w0 >> 32) : (uint32_t)w1,
-                       q2 = lo ? (uint32_t)w1 : (uint32_t)(w1 >> 32);
-        const uint32_t r0 = __funnelshift_r(q0, q1, s & 31u), r1 = __funnelshift_r(q1, q2, s & 31u);
-        // in stream order from the top, the first `need` of them
-        unsigned long long r = ((unsigned long long)__byte_perm(r0, 0, 0x0123) << 32) | __byte_perm(r1, 0, 0x0123);
-        r = need ? r & (~0ull << (64u - 8u * need)) : 0ull;
-        bb |= nbits < 64 ? r >> nbits : 0ull;
-        nbits += 8u * need;
-        pos += need;
-    };
-    topup();
-    // the state: bytes a0 .. a0 + 3, little-endian
-    uint32_t x = __byte_perm((uint32_t)(bb >> 32), 0, 0x0123);
-    bb <<= 32;
-    nbits -= 32;
-    const uint32_t* val32 = reinterpret_cast<const uint32_t*>(sm.val);
-    // SMALL: cumulative frequencies c1..c3 (M past the last symbol), frequencies and values
-    uint32_t c1 = 0, c2 = 0, c3 = 0, f0 = 0, f1 = 0, f2 = 0, f3 = 0;
-    T v0 = 0, v1 = 0, v2 = 0, v3 = 0;
-    if constexpr (SMALL) {
-        c1 = sm.cum[1];
-        c2 = c1 < zf::kAnsM ? sm.cum[2] : zf::kAnsM;
-        c3 = c2 < zf::kAnsM ? sm.cum[3] : zf::kAnsM;
-        const uint32_t c4 = c3 < zf::kAnsM ? sm.cum[4] : zf::kAnsM;
-        f0 = c1;
-        f1 = c2 - c1;
-        f2 = c3 - c2;
-        f3 = c4 - c3;
-        v0 = (T)sm.val[0];
-        v1 = c1 < zf::kAnsM ? (T)sm.val[1] : v0;
-        v2 = c2 < zf::kAnsM ? (T)sm.val[2] : v0;
-        v3 = c3 < zf::kAnsM ? (T)sm.val[3] : v0;
-    }
-    auto step = [&]() -> T {
-        T v;
-        if constexpr (SMALL) {
-            const uint32_t slot = x & (zf::kAnsM - 1u);
-            const bool b1 = slot >= c1, b2 = slot >= c2, b3 = slot >= c3;
-            const uint32_t c = b3 ? c3 : b2 ? c2 : b1 ? c1 : 0u;
-            const uint32_t f = b3 ? f3 : b2 ? f2 : b1 ? f1 : f0;
-            v = b3 ? v3 : b2 ? v2 : b1 ? v1 : v0;
-            x = f * (x >> zf::kAnsScale) + slot - c;
-        } else {
-            const uint32_t t = sm.slot[x & (zf::kAnsM - 1u)];
-            if constexpr (sizeof(T) == 4) v = (T)val32[2 * (t >> 24)];   // the low word of the 64-bit pattern
-            else v = (T)sm.val[t >> 24];
-            x = ((t & 0xFFFu) + 1u) * (x >> zf::kAnsScale) + ((t >> 12) & 0xFFFu);
+    uint4* ring = sm.ring[threadIdx.x];
+    const uint32_t* ring32 = reinterpret_cast<const uint32_t*>(ring);
+    const uint32_t end = ((a1 - 1) >> 4) + 1;             // 16-byte words [a0 >> 4, end) hold stream bytes (a1 > a0)
+    const uint32_t first = a0 >> 2;
+    uint32_t asked = (a0 >> 4) + kRing;                   // 16-byte words asked for (the first by ans_ask)
+    __pipeline_wait_prior(0);
+    auto load = [&](uint32_t i) { return ring32[i % (4 * kRing)]; };
+    uint32_t hi = __byte_perm(load(first), 0, 0x0123), lo = __byte_perm(load(first + 1), 0, 0x0123);
+    uint32_t next = first + 2, ahead = load(next);        // the word after the window
+    uint32_t used = 8u * (a0 & 3u);                       // bits of the window that have been taken
+    auto refill = [&]() {                                 // used < 64 -> used < 32
+        if (used >= 32u) {
+            hi = lo;
+            lo = __byte_perm(ahead, 0, 0x0123);
+            next++;
+            ahead = load(next);
         }
-        const uint32_t s = (x < zf::kAnsL ? 8u : 0u) + (x < (zf::kAnsL >> 8) ? 8u : 0u);
-        x = __funnelshift_l((uint32_t)(bb >> 32), x, s);
-        bb <<= s;
-        nbits -= s;
+        used &= 31u;
+    };
+    // before eight rows: the window's first byte lies in 16-byte word (next - 2) / 4
+    auto keep_ahead = [&]() {
+        if (asked < ((next - 2u) >> 2) + kRing) {
+            if (asked < end) __pipeline_memcpy_async(ring + asked % kRing, s2 + 16ull * asked, 16);
+            asked++;
+        }
+        __pipeline_commit();
+        __pipeline_wait_prior(1);
+    };
+    // the state: the first four bytes, little-endian
+    uint32_t x = __byte_perm(__funnelshift_l(lo, hi, used), 0, 0x0123);
+    used += 32;
+    refill();
+    const uint32_t* val32 = reinterpret_cast<const uint32_t*>(sm.val);
+    auto step = [&]() -> T {
+        const uint32_t t = sm.slot[x & (zf::kAnsM - 1u)], xh = x >> zf::kAnsScale;
+        const uint32_t sym = WIDE ? t >> 24 : (t >> 12) & 0x7Fu;
+        T v;
+        if constexpr (sizeof(T) == 4) v = (T)val32[2 * sym];   // the low word of the 64-bit pattern
+        else v = (T)sm.val[sym];
+        x = WIDE ? ((t >> 12) & 0xFFFu) * xh + (xh + (t & 0xFFFu)) : (t >> 19) * xh + (t & 0xFFFu);
+        const uint32_t s = x < (zf::kAnsL >> 8) ? 16u : x < zf::kAnsL ? 8u : 0u;
+        x = __funnelshift_l((uint32_t)(((((uint64_t)hi << 32) | lo) << used) >> 32), x, s);   // used < 48: its next 16 bits
+        used += s;
         return v;
     };
-    constexpr uint32_t V = 32 / sizeof(T);
+    constexpr uint32_t G = 8, V = 32 / sizeof(T);   // rows per step of the ring, rows per store
     const bool al32 = (reinterpret_cast<uintptr_t>(dst) & 31) == 0;
     uint32_t i0 = 0;
-    for (; i0 + V <= n; i0 += V) {
-        T v[V];
+    for (; i0 + G <= n; i0 += G) {
+        keep_ahead();
 #pragma unroll
-        for (uint32_t e = 0; e < V; e++) {
-            if (e % 4 == 0) topup();
-            v[e] = step();
-        }
-        if (al32) {
-            if constexpr (sizeof(T) == 4)
-                zfd::store32(dst + i0, ((unsigned long long)(uint32_t)v[1] << 32) | (uint32_t)v[0],
-                             ((unsigned long long)(uint32_t)v[3] << 32) | (uint32_t)v[2],
-                             ((unsigned long long)(uint32_t)v[5] << 32) | (uint32_t)v[4],
-                             ((unsigned long long)(uint32_t)v[7] << 32) | (uint32_t)v[6]);
-            else
-                zfd::store32(dst + i0, (uint64_t)v[0], (uint64_t)v[1], (uint64_t)v[2], (uint64_t)v[3]);
-        } else {
-            zfd::store_vec<T, V>(dst + i0, v);
+        for (uint32_t g = 0; g < G; g += V) {
+            T v[V];
+#pragma unroll
+            for (uint32_t e = 0; e < V; e += 2) {
+                v[e] = step();
+                v[e + 1] = step();
+                refill();
+            }
+            if (al32) {
+                if constexpr (sizeof(T) == 4)
+                    zfd::store32(dst + i0 + g, ((unsigned long long)(uint32_t)v[1] << 32) | (uint32_t)v[0],
+                                 ((unsigned long long)(uint32_t)v[3] << 32) | (uint32_t)v[2],
+                                 ((unsigned long long)(uint32_t)v[5] << 32) | (uint32_t)v[4],
+                                 ((unsigned long long)(uint32_t)v[7] << 32) | (uint32_t)v[6]);
+                else
+                    zfd::store32(dst + i0 + g, (uint64_t)v[0], (uint64_t)v[1], (uint64_t)v[2], (uint64_t)v[3]);
+            } else {
+                zfd::store_vec<T, V>(dst + i0 + g, v);
+            }
         }
     }
-    for (uint32_t e = 0; i0 < n; i0++, e++) {
-        if (e % 4 == 0) topup();
+    keep_ahead();
+    for (; i0 < n; i0++) {
         dst[i0] = step();
+        refill();
     }
-    const uint32_t used = (pos - a0) - nbits / 8;   // bytes the rows took
-    return used != a1 - a0 || x != zf::kAnsL;
+    __pipeline_wait_prior(0);
+    const uint32_t taken = 4u * (next - 2u - first) + used / 8u - (a0 & 3u);   // bytes the state and the rows took
+    return taken != a1 - a0 || x != zf::kAnsL;
+}
+
+// Ask for the first 16-byte words of a lane's stream.
+__device__ __forceinline__ void ans_ask(AnsSmem& sm, const uint8_t* s2, uint32_t a0, uint32_t a1) {
+    const uint32_t w = a0 >> 4, end = ((a1 - 1) >> 4) + 1;
+    for (uint32_t i = w; i < w + kRing; i++)
+        if (i < end) __pipeline_memcpy_async(sm.ring[threadIdx.x] + i % kRing, s2 + 16ull * i, 16);
+    __pipeline_commit();
+}
+
+// Slot entries: warp w fills the ranges of symbols w, w + kWarps, ..., a range's
+// slots side by side over the lanes.  (A contiguous 32 slots per thread, each
+// thread walking its symbols, took 4 to 8 us more of a call.)
+template <bool WIDE>
+__device__ __forceinline__ void ans_table(AnsSmem& sm, uint32_t nd, uint32_t lane, uint32_t warp) {
+    for (uint32_t s = warp; s < nd; s += kWarps) {
+        const uint32_t c = sm.cum[s], f = sm.cum[s + 1] - c;
+        for (uint32_t d = lane; d < f; d += 32) sm.slot[c + d] = ans_entry<WIDE>(s, f, d);
+    }
 }
 
 // The CTA builds its chunk's tables, then warp w decodes job blockIdx.x *
@@ -177,6 +202,19 @@ __global__ void __launch_bounds__(kWarps * 32) ans_kernel(const __grid_constant_
         if (tid == 0) zfd::report(err, ZF_ECORRUPT, c.chunk_id);
         return;   // uniform over the CTA
     }
+    // one stream per lane; its first bytes are on their way while the tables are built
+    const uint32_t job = job0 + warp;
+    const uint32_t k = (job - c.tile0) * zf::kAnsStreamsPerJob + lane;
+    const uint8_t* s2 = c.blob + h.off[2];
+    uint32_t a0 = 0, a1 = 0;
+    bool bad = false;
+    if (k < K) {
+        const uint32_t* starts = reinterpret_cast<const uint32_t*>(c.blob + h.off[1] + fb);
+        a0 = __ldg(starts + k);
+        a1 = __ldg(starts + k + 1);
+        bad = a1 < a0 || a1 - a0 < 4u || a1 > h.len[2];
+        if (!bad) ans_ask(sm, s2, a0, a1);
+    }
     // frequencies, two per thread, and their exclusive scan over the CTA
     const uint16_t* fq = reinterpret_cast<const uint16_t*>(c.blob + h.off[1]);
     const uint32_t i0 = 2 * tid;
@@ -193,6 +231,7 @@ __global__ void __launch_bounds__(kWarps * 32) ans_kernel(const __grid_constant_
         total += sm.wsum[q];
     }
     if (__syncthreads_or(fbad) || total != zf::kAnsM) {
+        __pipeline_wait_prior(0);
         if (tid == 0) zfd::report(err, ZF_ECORRUPT, c.chunk_id);
         return;
     }
@@ -204,46 +243,15 @@ __global__ void __launch_bounds__(kWarps * 32) ans_kernel(const __grid_constant_
         sm.val[k] = sz == 8 ? (unsigned long long)__ldg(reinterpret_cast<const int64_t*>(c.blob + h.off[0]) + k)
                             : (unsigned long long)(uint32_t)__ldg(reinterpret_cast<const int32_t*>(c.blob + h.off[0]) + k);
     __syncthreads();
-    // slot entries: thread t fills slots [t * 32, t * 32 + 32), walking the
-    // symbols from the one holding its first slot (binary search on cum);
-    // chunks of at most four values decode from the cumulative frequencies
-    if (nd > 4) {
-        constexpr uint32_t per = zf::kAnsM / (kWarps * 32);
-        const uint32_t first = tid * per;
-        uint32_t lo = 0, hi = nd - 1;   // the last symbol whose cum is <= first
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (sm.cum[mid] <= first) lo = mid;
-            else hi = mid - 1;
-        }
-        uint32_t s = lo, cs = sm.cum[s], ce = sm.cum[s + 1];
-        for (uint32_t slot = first; slot < first + per; slot++) {
-            while (slot >= ce) {
-                s++;
-                cs = ce;
-                ce = sm.cum[s + 1];
-            }
-            sm.slot[slot] = (s << 24) | ((slot - cs) << 12) | (ce - cs - 1u);
-        }
-    }
+    if (nd > 128) ans_table<true>(sm, nd, lane, warp);
+    else ans_table<false>(sm, nd, lane, warp);
     __syncthreads();
-    // one stream per lane
-    const uint32_t job = job0 + warp;
-    const uint32_t k = (job - c.tile0) * zf::kAnsStreamsPerJob + lane;
-    bool bad = false;
-    if (k < K) {
-        const uint32_t* starts = reinterpret_cast<const uint32_t*>(c.blob + h.off[1] + fb);
-        const uint32_t a0 = __ldg(starts + k), a1 = __ldg(starts + k + 1);
+    if (k < K && !bad) {
         const uint32_t r0 = k * L, n = min(L, h.rows - r0);
-        if (a1 < a0 || a1 - a0 < 4u || a1 > h.len[2]) {
-            bad = true;
-        } else if (sz == 8) {
-            bad = nd <= 4 ? ans_stream<int64_t, true>(sm, c.blob + h.off[2], a0, a1, reinterpret_cast<int64_t*>(c.dst) + r0, n)
-                          : ans_stream<int64_t, false>(sm, c.blob + h.off[2], a0, a1, reinterpret_cast<int64_t*>(c.dst) + r0, n);
-        } else {
-            bad = nd <= 4 ? ans_stream<int32_t, true>(sm, c.blob + h.off[2], a0, a1, reinterpret_cast<int32_t*>(c.dst) + r0, n)
-                          : ans_stream<int32_t, false>(sm, c.blob + h.off[2], a0, a1, reinterpret_cast<int32_t*>(c.dst) + r0, n);
-        }
+        int32_t* d4 = reinterpret_cast<int32_t*>(c.dst) + r0;
+        int64_t* d8 = reinterpret_cast<int64_t*>(c.dst) + r0;
+        if (sz == 8) bad = nd > 128 ? ans_stream<int64_t, true>(sm, s2, a0, a1, d8, n) : ans_stream<int64_t, false>(sm, s2, a0, a1, d8, n);
+        else bad = nd > 128 ? ans_stream<int32_t, true>(sm, s2, a0, a1, d4, n) : ans_stream<int32_t, false>(sm, s2, a0, a1, d4, n);
     }
     if (bad) zfd::report(err, ZF_ECORRUPT, c.chunk_id);
 }
