@@ -1025,6 +1025,7 @@ zf_status parse_serialized(zf_compressed* c, std::string* why) {
             expect += ch.bytes;
             if (!check_chunk(h + ch.off, ch.bytes, pi.scheme, pi.dtype, ch.rows, &ch.bmax, why)) return ZF_ECORRUPT;
             if (pi.scheme == ZF_STRDICT || pi.scheme == ZF_ANS) ch.units = (uint32_t)rd<uint64_t>(h + ch.off + 16);
+            if (pi.scheme == ZF_STRDICT) ch.dict_bytes = rd<uint32_t>(h + ch.off + 40) + 7u * rd<uint32_t>(h + ch.off + 12);
             ch.off += pos;
             ch.scheme = (uint8_t)pi.scheme;
             ch.dtype = (uint8_t)pi.dtype;

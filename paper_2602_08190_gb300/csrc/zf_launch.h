@@ -56,6 +56,12 @@ uint32_t warp_smem_bytes(int scheme, int dtype, uint32_t bmax);
 cudaError_t launch_tiles(const TileLaunch& L, cudaStream_t s);
 cudaError_t launch_lz(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t n, uint32_t* err, int num_sms, cudaStream_t s);
 cudaError_t launch_lz_cta(const ChunkArgs& chunks, uint32_t* err, cudaStream_t s);
+// String-dictionary chunks whose dictionaries take at most dict_bytes
+// (ChunkInfo::dict_bytes, at most strdict_smem_limit()) of shared memory;
+// descriptors carry tile0 and ntiles in 1024-token tiles.
+uint32_t strdict_smem_limit();
+cudaError_t launch_strdict(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t nchunks, uint32_t ntiles,
+                           uint32_t dict_bytes, uint32_t* err, int num_sms, cudaStream_t s);
 // ANS chunks: njobs warp jobs of up to 32 streams (chunk descriptors carry tile0 in jobs).
 cudaError_t launch_ans(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t nchunks, uint32_t njobs, uint32_t* err,
                        cudaStream_t s);

@@ -244,7 +244,23 @@ struct Group {
     uint32_t warp_smem;  // widest per-warp shared memory of the group's chunks
     uint32_t tile_rows;  // rows of a warp job in this launch
     uint32_t threads;    // threads per CTA of this launch
+    uint32_t dict_bytes; // kStrdictSmem: most shared memory a chunk's dictionary takes
 };
+
+// Group::scheme of string-dictionary chunks whose dictionary fits in shared
+// memory beside the warps' windows (197,632 bytes: 13,000 entries of 8 bytes,
+// say; zf_strdict_sm.cu); a larger one is read through L1 (zf_strdict.cuh).
+constexpr int kStrdictSmem = ZF_NSCHEMES;
+
+// The launch a chunk belongs to: LZ77, ANS and string dictionaries in shared
+// memory have kernels of their own, batched or not.
+std::pair<int, int> group_key(const zf::ChunkInfo& ch, bool batched) {
+    if (ch.scheme == ZF_LZ77) return {ZF_LZ77, ZF_BYTES};
+    if (ch.scheme == ZF_ANS) return {ch.scheme, ch.dtype};
+    if (batched) return {-1, -1};
+    if (ch.scheme == ZF_STRDICT && ch.dict_bytes <= zf::strdict_smem_limit()) return {kStrdictSmem, ZF_BYTES};
+    return {ch.scheme, ch.dtype};
+}
 
 // Append descriptors of works[b, e) to `desc`, grouped for launching.
 void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_t e, const zf_kcfg& k,
@@ -252,34 +268,26 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
     const bool batched = k.flags & ZF_KCFG_BATCHED;
     std::vector<std::pair<int, int>> keys;
     for (size_t i = b; i < e; i++) {
-        int s = w[i].ch->scheme, d = w[i].ch->dtype;
-        if (s == ZF_LZ77) {
-            d = ZF_BYTES;
-        } else if (s == ZF_ANS) {
-            // ANS streams have their own kernel, batched or not
-        } else if (batched) {
-            s = -1;
-            d = -1;
-        }
-        if (std::find(keys.begin(), keys.end(), std::make_pair(s, d)) == keys.end()) keys.push_back({s, d});
+        const auto key = group_key(*w[i].ch, batched);
+        if (std::find(keys.begin(), keys.end(), key) == keys.end()) keys.push_back(key);
     }
     for (auto& key : keys) {
         uint32_t bmax = 0;   // widest bit width of the group: its geometry class
         uint64_t units = 0;  // rows (string dictionary: tokens) of the group
+        uint32_t dict_bytes = 0;
         for (size_t i = b; i < e; i++) {
             const zf::ChunkInfo& ch = *w[i].ch;
-            if (ch.scheme == key.first && ch.dtype == key.second) bmax = std::max<uint32_t>(bmax, ch.bmax);
-            if (key.first < 0 ? ch.scheme != ZF_LZ77 && ch.scheme != ZF_ANS : ch.scheme == key.first && ch.dtype == key.second)
-                units += ch.scheme == ZF_STRDICT ? ch.units : ch.rows;
+            if (group_key(ch, batched) != key) continue;
+            if (key.first >= 0) bmax = std::max<uint32_t>(bmax, ch.bmax);
+            units += ch.scheme == ZF_STRDICT ? ch.units : ch.rows;
+            dict_bytes = std::max(dict_bytes, ch.dict_bytes);
         }
-        const Geometry geo = group_geometry(ctx, k, key.first, key.second, bmax, units);
-        Group g{key.first, key.second, (uint32_t)desc.size(), 0, 0, 16, geo.tile_rows, geo.threads};
+        const Geometry geo = key.first == kStrdictSmem ? Geometry{zf::kStrTile, 0}
+                                                       : group_geometry(ctx, k, key.first, key.second, bmax, units);
+        Group g{key.first, key.second, (uint32_t)desc.size(), 0, 0, 16, geo.tile_rows, geo.threads, dict_bytes};
         for (size_t i = b; i < e; i++) {
-            int s = w[i].ch->scheme, d = w[i].ch->dtype;
-            bool lz = s == ZF_LZ77, own = lz || s == ZF_ANS;   // chunks with a kernel of their own
-            bool match = lz ? key.first == ZF_LZ77
-                            : (key.first < 0 ? true : (key.first == s && key.second == d));
-            if (!match || (key.first < 0 && own)) continue;
+            const int s = w[i].ch->scheme, d = w[i].ch->dtype;
+            if (group_key(*w[i].ch, batched) != key) continue;
             ZfDevChunk dc{};
             dc.blob = w[i].dev;
             dc.dst = w[i].dst;
@@ -318,6 +326,8 @@ zf_status launch_groups(zf_ctx* ctx, const Group* groups, size_t ngroups, const 
         cudaError_t e;
         if (g.scheme == ZF_LZ77) {
             e = zf::launch_lz(dchunks, hchunks, g.count, ctx->d_errw, ctx->num_sms, stream);
+        } else if (g.scheme == kStrdictSmem) {
+            e = zf::launch_strdict(dchunks, hchunks, g.count, g.ntiles, g.dict_bytes, ctx->d_errw, ctx->num_sms, stream);
         } else if (g.scheme == ZF_ANS) {
             e = zf::launch_ans(dchunks, hchunks, g.count, g.ntiles, ctx->d_errw, stream);
         } else {
