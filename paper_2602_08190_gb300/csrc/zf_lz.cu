@@ -40,11 +40,10 @@ constexpr uint32_t kLzWin = 4096;      // batch output window per warp
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 // Launches of at most this many blocks per SM take a CTA per block
 // (zf_lz_cta.cu).  A warp takes 540 us for a block of text however few there
-// are, a CTA per block adds 0.32 us for each block to about 60 us: resident
-// calls of 8, 64, 128 and 160 MB took 100, 387, 726 and 870 us with a CTA and
-// 568, 681, 791 and 848 us with a warp per block (2,432 blocks, 16 per SM,
-// would be even).
-constexpr uint32_t kLzCtaBlocksPerSm = 14;
+// are, a CTA per block adds 0.3 us for each block to about 60 us: resident
+// calls of 16, 64 and 128 MB took 118, 368 and 683 us with a CTA and 578, 681
+// and 785 us with a warp per block; 160 MB, 17 blocks per SM, would be even.
+constexpr uint32_t kLzCtaBlocksPerSm = 15;
 
 struct LzParse {
     uint32_t vp = 0;        // next byte of the lengths stream

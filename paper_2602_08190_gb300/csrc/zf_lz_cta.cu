@@ -41,9 +41,12 @@ namespace {
 //   global memory.
 // What bounds it: the latency of a batch's chain of barriers, scans and
 // shared-memory lookups (14 batches of text per block).  Among thousands of
-// blocks it is bound by issue slots, 234,000 warp instructions per block of
-// text.  Measured on GB300: 21 blocks of text (1.3 MB) 94 us per call with
-// its host part, 540 us with one warp per block.
+// blocks it is bound by issue slots (64% busy), 228,000 warp instructions per
+// block of text: 40% of them to parse, place and store tokens, the rest in
+// about equal parts shortcuts with lookups of bytes.  Measured on GB300: 21
+// blocks of text (1.3 MB) 87 us per call with its host part, 548 us with one
+// warp per block; 1,024 blocks 368 and 681 us.  Shortcuts whose steps were not
+// left for other tokens cost 27 us more of the 368.
 constexpr uint32_t kLzThreads = 512;
 constexpr uint32_t kLzWarps = kLzThreads / 32;
 constexpr uint32_t kLzRing = 4096;             // parsed lengths: at most 1,023 left over and 2,048 more
@@ -54,9 +57,9 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kDone = 0x8000u;            // state of a byte: kDone | value, or the position it copies
 
 struct LzSmem {
-    uint8_t out[zf::kLzBlock];            // the block's output
     uint2 st[kLzSeg / 4];                 // states of the segment's bytes, four 16-bit states per word
-    uint8_t lit[kLzLit];                  // literal byte i of s2 at i mod kLzLit
+    uint8_t out[zf::kLzBlock];            // the block's output (a lookup may read three bytes on either side)
+    uint8_t lit[kLzLit + 16];             // literal byte i of s2 at i mod kLzLit; the first 16 again at the end
     uint2 tok[kLzThreads];                // x = last byte before the match | offset << 16,
                                           // y = output minus literal position | last byte << 16
     uint2 starts[kLzSeg / 32];            // x = token starts in 32 bytes, y = tokens of the batch that start before them
@@ -107,27 +110,55 @@ __device__ __forceinline__ uint2 lz_lookup(const LzSmem& sm, const uint8_t* __re
     const uint32_t pb = nib ? __ffs(nib) - 1 : 4u;
     const uint2 ta = sm.tok[n ? n - 1 : 0];
     const uint2 tb = nib ? sm.tok[n] : ta;
-    constexpr uint32_t OUT = offsetof(LzSmem, out), LIT = offsetof(LzSmem, lit);
-    const uint8_t* smb = reinterpret_cast<const uint8_t*>(&sm);
     uint32_t v[4];
+    if constexpr (RING) {
+        // per token: the byte 0 of the word as a literal and as a copy, one address each
+        constexpr uint32_t OUT = offsetof(LzSmem, out), LIT = offsetof(LzSmem, lit);
+        const uint8_t* smb = reinterpret_cast<const uint8_t*>(&sm);
+        const uint32_t la = ta.x & 0xFFFFu, lb = tb.x & 0xFFFFu, oa = ta.x >> 16, ob = tb.x >> 16;
+        const int ma = (int)(j0 - oa), mb = (int)(j0 - ob);   // -3 or more where a byte of the segment copies from them
+        const uint32_t ka = LIT + ((j0 - (ta.y & 0xFFFFu)) & (kLzLit - 1)), kb = LIT + ((j0 - (tb.y & 0xFFFFu)) & (kLzLit - 1));
+        bool over = false;   // a byte that copies its own match's output
 #pragma unroll
-    for (uint32_t b = 0; b < 4; b++) {
-        const uint32_t j = j0 + b;
-        const uint2 t = b >= pb ? tb : ta;
-        const uint32_t last = t.x & 0xFFFFu, off = t.x >> 16;
-        const bool in = j >= s0 && j < s1, is_lit = j <= last;
-        uint32_t src = j - off;
-        if (!is_lit && src > last && in) src = last + 1 - off + (j - last - 1) % off;   // overlaps its own output
-        const uint32_t li = j - (t.y & 0xFFFFu);
-        const bool here = in && !is_lit && src >= s0;   // copies a byte of this segment
-        if constexpr (RING) {
-            const uint32_t x = smb[is_lit ? LIT + (li & (kLzLit - 1)) : OUT + (src & (zf::kLzBlock - 1))];
-            v[b] = here ? src - base : kDone | x;
-        } else {
-            uint32_t x = 0;
-            if (in && is_lit) x = __ldg(lit + li);
-            else if (in && !here) x = sm.out[src];
-            v[b] = here ? src - base : kDone | x;
+        for (uint32_t b = 0; b < 4; b++) {
+            const bool second = b >= pb;
+            const uint32_t last = second ? lb : la, k = second ? kb : ka;
+            const int m = second ? mb : ma;
+            const bool is_lit = j0 + b <= last, here = !is_lit && m + (int)b >= (int)s0;
+            over |= !is_lit && m + (int)b > (int)last;
+            const uint32_t x = smb[(is_lit ? k : OUT + (uint32_t)max(m, -3)) + b];
+            v[b] = here ? (uint32_t)m + b - base : kDone | x;
+        }
+        if (over) {
+#pragma unroll
+            for (uint32_t b = 0; b < 4; b++) {
+                const bool second = b >= pb;
+                const uint32_t last = second ? lb : la, off = second ? ob : oa, j = j0 + b;
+                if (j <= last || j - off <= last || j < s0 || j >= s1) continue;
+                const uint32_t src = last + 1 - off + (j - last - 1) % off;
+                v[b] = src >= s0 ? src - base : kDone | sm.out[src];
+            }
+        }
+        if (j0 < s0 || j0 + 4 > s1) {   // bytes outside the segment: nothing copies them
+#pragma unroll
+            for (uint32_t b = 0; b < 4; b++)
+                if (j0 + b < s0 || j0 + b >= s1) v[b] = kDone;
+        }
+    } else {
+#pragma unroll
+        for (uint32_t b = 0; b < 4; b++) {
+            const uint32_t j = j0 + b;
+            const uint2 t = b >= pb ? tb : ta;
+            const uint32_t last = t.x & 0xFFFFu, off = t.x >> 16;
+            v[b] = kDone;
+            if (j < s0 || j >= s1) continue;
+            if (j <= last) {
+                v[b] = kDone | __ldg(lit + (j - (t.y & 0xFFFFu)));
+            } else {
+                uint32_t src = j - off;
+                if (src > last) src = last + 1 - off + (j - last - 1) % off;
+                v[b] = src >= s0 ? src - base : kDone | sm.out[src];
+            }
         }
     }
     return make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
@@ -137,8 +168,10 @@ __device__ __forceinline__ uint2 lz_lookup(const LzSmem& sm, const uint8_t* __re
 // asks for the 16-byte words from `have` on and returns the new `have`.
 __device__ __forceinline__ uint32_t lz_fill(LzSmem& sm, const uint8_t* lit, uint32_t l2, uint32_t from, uint32_t have) {
     const uint32_t to = min((l2 + 15) & ~15u, (from & ~15u) + kLzLit);
-    for (uint32_t i = have + 16 * threadIdx.x; i < to; i += 16 * kLzThreads)
+    for (uint32_t i = have + 16 * threadIdx.x; i < to; i += 16 * kLzThreads) {
         __pipeline_memcpy_async(sm.lit + (i & (kLzLit - 1)), lit + i, 16);
+        if ((i & (kLzLit - 1)) == 0) __pipeline_memcpy_async(sm.lit + kLzLit, lit + i, 16);
+    }
     __pipeline_commit();
     return max(have, to);
 }
@@ -235,11 +268,14 @@ __device__ void lz_block(const ZfDevChunk& c, LzSmem& sm, uint32_t* err) {
         const uint32_t ll = pair & 0xFFFFu, ml = has_m ? (pair >> 16) + zf::kLzMinMatch : 0;
         const uint32_t off = has_m ? off_next : 0;
         off_next = t + kLzThreads + 1 < T ? __ldg(offs + t + kLzThreads) : 0;
-        uint32_t lend = ll, oend = ll + ml;                  // at most 512 * 2^17: no sum wraps
-#pragma unroll
-        for (uint32_t d = 1; d < 32; d <<= 1) {
-            const uint32_t a = __shfl_up_sync(kFull, lend, d), b = __shfl_up_sync(kFull, oend, d);
-            if (lane >= d) { lend += a; oend += b; }
+        uint32_t lend, oend;                                 // inclusive sums over the lanes
+        if (!__any_sync(kFull, ll + ml >= 2048u)) {          // both below 2^16: one scan
+            const uint32_t both = zfd::warp_incl_sum<uint32_t>(ll | ((ll + ml) << 16), lane);
+            lend = both & 0xFFFFu;
+            oend = both >> 16;
+        } else {                                             // at most 512 * 2^17 over the CTA: no sum wraps
+            lend = zfd::warp_incl_sum<uint32_t>(ll, lane);
+            oend = zfd::warp_incl_sum<uint32_t>(ll + ml, lane);
         }
         if (lane == 31) {
             sm.wl[warp] = lend;
@@ -270,7 +306,8 @@ __device__ void lz_block(const ZfDevChunk& c, LzSmem& sm, uint32_t* err) {
             }
             if (__syncthreads_or(bad)) { ok = false; break; }
             if (has_m && mpos < s1 && oend > s0) {
-                // the source lies inside one match of this segment: copy what that match copies
+                // the source lies inside one match of this segment: copy what that match copies; every step is
+                // left for the tokens that look here, so a chain of n matches takes about log2 n steps
                 uint32_t o = off;
                 for (;;) {
                     const uint32_t src = mpos - o;
@@ -280,8 +317,8 @@ __device__ void lz_block(const ZfDevChunk& c, LzSmem& sm, uint32_t* err) {
                     const uint32_t ux = *const_cast<const volatile uint32_t*>(&u->x);   // its owner may shorten it meanwhile
                     if (src <= (ux & 0xFFFFu) || src + ml - 1 > (u->y >> 16)) break;
                     o += ux >> 16;
+                    *reinterpret_cast<volatile uint32_t*>(&sm.tok[tid].x) = (mpos - 1) | (o << 16);
                 }
-                if (o != off) *reinterpret_cast<volatile uint32_t*>(&sm.tok[tid].x) = (mpos - 1) | (o << 16);
             }
             __pipeline_wait_prior(0);
             __syncthreads();
