@@ -14,11 +14,10 @@
 //               16-byte store (coalesced).  Float2Int makes each integer
 //               the double nearest d / 10^e with integer multiplies
 //               (zf_f2i.h) and then patches the chunk's exceptions.
-//   delta_job   Group-Parallel: one 1024-row block per step.  Lane l owns
-//               values [32l, 32l+32): it sums its differences, one warp
-//               shuffle scan gives every lane its offset, the values are
-//               rebuilt from a second read of the differences and leave
-//               through a shared-memory transpose, four lanes per 128-byte line.
+//   delta_job   Group-Parallel: one 1024-row block at a time, 128 values per
+//               step: every lane extracts four differences, a warp shuffle
+//               scan of their sums places them, and the values leave with one
+//               coalesced vector store per lane.
 //   rle_job     Group-Parallel: the tile's run lengths (the chunk's 1024-row
 //               directory names the first run) are scanned into start rows,
 //               four per lane and one warp shuffle scan per 128 runs (the
@@ -93,7 +92,7 @@ __device__ __forceinline__ uint64_t extract(const uint32_t* sm, uint32_t bitpos,
 // it are inlined into their kernels (the batched kernel included): inside a
 // function called out of line (through the ABI) the same store was seen to
 // write only its first word on sm_103a, so no out-of-line function uses it
-// (WS = false in delta_block_wide).
+// (delta_block_wide).
 __device__ __forceinline__ void store32(void* dst, unsigned long long a, unsigned long long b, unsigned long long c,
                                         unsigned long long d) {
     const size_t g = __cvta_generic_to_global(dst);
@@ -372,148 +371,39 @@ __device__ void fp_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t 
 }
 
 // ---------------------------------------------------------------- delta (Group-Parallel)
-// Swizzle of the 16-byte chunks of a lane's 128-byte line in the transpose
-// buffer: x = 4a + c (a < 2, c < 4) -> 2c + a.  Eight consecutive lanes
-// writing chunk k land in eight different bank groups, and so do the eight
-// lanes of a read phase (two lane quads reading the even or the odd chunks of
-// owners 4 apart, whose swizzles differ in parity).
-__device__ __forceinline__ uint32_t xswz(uint32_t l) {
-    l &= 7;
-    return ((l & 3) << 1) | (l >> 2);
-}
-
-// Stores of lane-owned lines, four lanes per line: every lane has put its
-// 128-byte line (eight 16-byte chunks, swizzled) in `xb`; in step r the lanes
-// of quad q write the four 32-byte sectors of lane 4q + r's line, so each
-// 256-bit store instruction writes eight whole 128-byte lines instead of 32
-// single sectors of 32 lines (the L2 takes a quarter of the requests).
-// `line0` is lane 0's line; lane o's is line0 + o * lane_bytes.
-__device__ __forceinline__ void store_lines_x4(char* line0, uint32_t lane_bytes, const uint4* xb, uint32_t lane) {
-    const uint32_t q4 = lane & ~3u, i4 = lane & 3u;
-#pragma unroll
-    for (uint32_t r = 0; r < 4; r++) {
-        const uint32_t o = q4 + r, fo = xswz(o);
-        const uint4 a = xb[o * 8 + ((2 * i4) ^ fo)], c = xb[o * 8 + ((2 * i4 + 1) ^ fo)];
-        store32(line0 + o * lane_bytes + 32 * i4, ((unsigned long long)a.y << 32) | a.x,
-                ((unsigned long long)a.w << 32) | a.z, ((unsigned long long)c.y << 32) | c.x,
-                ((unsigned long long)c.w << 32) | c.z);
-    }
-}
-
-// One 1024-row block with each lane owning 32 consecutive values
-// [32*lane, 32*lane + 32): a single warp scan per block.  The lane's bits
-// start on a word boundary (32*lane*b bits = lane*b words), so every lane
-// walks the same bit positions and the refill of the two-word bit reader is
-// uniform across the warp.  The lane's differences are read twice: once for
-// their sum (the warp scan needs it first), once to rebuild the values, so no
-// array of prefixes stays live in registers.  Full blocks at a 32-byte
-// aligned address leave through the transpose buffer `xb` (4 KiB per warp),
-// four lanes per 128-byte line (store_lines_x4); other blocks in 32-byte
-// stores (four int64 or eight int32), each a whole L2 sector.  WIDE
-// (b > 21): 64-bit sums and funnel-shift extraction; otherwise 32-bit sums
-// (32 * 1024 * (2^21 - 1) < 2^32).
-template <class T, bool WIDE, bool WS>
+// A block of differences of more than 21 bits: 64-bit sums.  Each lane owns 32
+// consecutive values [32*lane, 32*lane + 32): it sums its differences, one warp
+// scan gives every lane its offset, and the values are rebuilt from a second
+// extraction, so no array of prefixes stays live in registers.
+template <class T>
 __device__ __forceinline__ void delta_block_lanes(T* dst, const uint32_t* wsm, uint32_t mk, uint32_t b, uint64_t base,
-                                                  uint64_t min_d, uint32_t lane, uint4* xb) {
+                                                  uint64_t min_d, uint32_t lane) {
     using U = typename std::conditional<sizeof(T) == 8, unsigned long long, unsigned int>::type;
-    using S = typename std::conditional<WIDE, unsigned long long, unsigned int>::type;
     constexpr int PER = 32 / sizeof(T);           // values per 32-byte store
     const uint32_t j0 = lane * 32;
     const uint32_t nv = mk > j0 ? min(32u, mk - j0) : 0u;   // valid values of this lane
-    const uint32_t mask = WIDE ? 0u : (1u << b) - 1u;
-    // bit reader over the lane's differences (narrow: two words in registers)
-    uint32_t wi = 0, lo = 0, hi = 0, pos = 0;
-    auto start = [&]() {
-        if constexpr (!WIDE) {
-            wi = lane * b;
-            lo = wsm[wi];
-            hi = wsm[wi + 1];
-            wi += 2;
-            pos = 0;
-        }
-    };
     // difference k of the lane (u_0 of the block and slots past the block count as 0)
-    auto diff = [&](uint32_t k, bool full) -> S {
-        S u;
-        if constexpr (!WIDE) {
-            u = __funnelshift_r(lo, hi, pos) & mask;
-            pos += b;
-            if (pos >= 32) {
-                lo = hi;
-                hi = wsm[wi++];
-                pos -= 32;
-            }
-        } else {
-            u = (full || k < nv) ? (S)extract(wsm, (j0 + k) * b, b) : (S)0;
-        }
-        if ((!full && k >= nv) || (k == 0 && lane == 0)) u = 0;
-        return u;
+    auto diff = [&](uint32_t k) -> unsigned long long {
+        return k >= nv || (k == 0 && lane == 0) ? 0ull : extract(wsm, (j0 + k) * b, b);
     };
-    start();
-    S total = 0;
+    unsigned long long total = 0;
 #pragma unroll
-    for (uint32_t k = 0; k < 32; k++) total += diff(k, false);
-    const S excl = warp_incl_sum<S>(total, lane) - total;
+    for (uint32_t k = 0; k < 32; k++) total += diff(k);
+    const unsigned long long excl = warp_incl_sum<unsigned long long>(total, lane) - total;
     const U md = (U)min_d;
     // x_{j0+k} = base + (j0 + k) * min_d + (differences up to j0 + k): acc after
     // step k, where each step adds min_d + u_k
     U acc = (U)base + (U)j0 * md + (U)excl - md;
-    start();
-    const bool al32 = WS && (reinterpret_cast<uintptr_t>(dst + j0) & 31) == 0;
-    if constexpr (WS && !WIDE) {
-        if (al32 && mk == zf::kDeltaBlock) {   // warp-uniform: dst is the block's first row
-            constexpr uint32_t LANE_BYTES = 32 * sizeof(T), LINES = LANE_BYTES / 128;
-            const uint32_t f = xswz(lane);
-#pragma unroll
-            for (uint32_t h = 0; h < LINES; h++) {
-#pragma unroll
-                for (uint32_t k8 = 0; k8 < 8; k8++) {
-                    uint4 w;
-                    if constexpr (sizeof(T) == 8) {
-                        const uint32_t k = h * 16 + k8 * 2;
-                        acc += md + (U)diff(k, true);
-                        const U v0 = acc;
-                        acc += md + (U)diff(k + 1, true);
-                        w = make_uint4((uint32_t)v0, (uint32_t)(v0 >> 32), (uint32_t)acc, (uint32_t)(acc >> 32));
-                    } else {
-                        uint32_t a[4];
-#pragma unroll
-                        for (uint32_t e = 0; e < 4; e++) {
-                            acc += md + (U)diff(k8 * 4 + e, true);
-                            a[e] = (uint32_t)acc;
-                        }
-                        w = make_uint4(a[0], a[1], a[2], a[3]);
-                    }
-                    xb[lane * 8 + (k8 ^ f)] = w;
-                }
-                __syncwarp();
-                store_lines_x4(reinterpret_cast<char*>(dst) + h * 128, LANE_BYTES, xb, lane);
-                __syncwarp();
-            }
-            return;
-        }
-    }
 #pragma unroll
     for (int q = 0; q < 32 / PER; q++) {
         T v[PER];
 #pragma unroll
         for (int e = 0; e < PER; e++) {
-            acc += md + (U)diff(q * PER + e, false);
+            acc += md + (U)diff(q * PER + e);
             v[e] = (T)acc;
         }
         if ((uint32_t)(q * PER + PER) <= nv) {
-            if (WS && al32) {
-                if constexpr (sizeof(T) == 8) {
-                    store32(dst + j0 + q * PER, (uint64_t)v[0], (uint64_t)v[1], (uint64_t)v[2], (uint64_t)v[3]);
-                } else {
-                    store32(dst + j0 + q * PER, ((uint64_t)(uint32_t)v[1] << 32) | (uint32_t)v[0],
-                            ((uint64_t)(uint32_t)v[3] << 32) | (uint32_t)v[2],
-                            ((uint64_t)(uint32_t)v[5] << 32) | (uint32_t)v[4],
-                            ((uint64_t)(uint32_t)v[7] << 32) | (uint32_t)v[6]);
-                }
-            } else {
-                store_vec<T, PER>(dst + j0 + q * PER, v);
-            }
+            store_vec<T, PER>(dst + j0 + q * PER, v);
         } else {
 #pragma unroll
             for (int e = 0; e < PER; e++)
@@ -522,14 +412,84 @@ __device__ __forceinline__ void delta_block_lanes(T* dst, const uint32_t* wsm, u
     }
 }
 
-// Blocks of more than 21 bits per difference are rare; out of line, they do
-// not add to the registers of the common path.  They keep 16-byte stores: in
-// an out-of-line function a 256-bit store from inline PTX wrote only part of
-// its data (seen on GB300; the same store inlined is exact).
+// Four consecutive differences of b bits from bit `pos` of the staged words.
+// W = 1: b <= 8, all four in one window of two words; W = 2: b <= 16, two in
+// each window; W = 4: one.
+template <int W>
+__device__ __forceinline__ void delta_diffs(const uint32_t* wsm, uint32_t pos, uint32_t b, uint32_t mask, uint32_t (&u)[4]) {
+    constexpr int PER = 4 / W;
+#pragma unroll
+    for (int g = 0; g < W; g++) {
+        const uint32_t p = pos + g * PER * b, w = p >> 5, sh = p & 31;
+        const uint32_t w0 = wsm[w], w1 = wsm[w + 1];
+        const uint32_t lo = __funnelshift_r(w0, w1, sh), hi = w1 >> sh;
+#pragma unroll
+        for (int k = 0; k < PER; k++) u[g * PER + k] = (k ? __funnelshift_r(lo, hi, k * b) : lo) & mask;   // k * b <= 24
+    }
+}
+
+// A block of differences of at most 21 bits (32-bit sums: 1024 * (2^21 - 1) <
+// 2^31), 128 values per step: lane l takes four consecutive differences, one
+// warp scan of the lanes' sums places them, and the values leave with one
+// coalesced 16- or 32-byte store per lane.  OFF32: base + j * min_d + sum fits
+// 32 bits past the base (the caller has checked), so a 64-bit value is one
+// 32-bit multiply-add and one 64-bit add.
+// What bounds it: DRAM for int64 (64M rows, gaps of mean 4: 108 us per resident
+// call, 6.0 TB/s over its kernel), the issue of 27 instructions a row and the
+// scans' latency for int32 (77 us).  Lanes that owned 32 consecutive values,
+// extracted them twice and turned them in shared memory took 39 instructions a
+// row, 117 and 96 us.
+template <class T, int W, bool OFF32>
+__device__ __forceinline__ void delta_block(T* dst, const uint32_t* wsm, uint32_t mk, uint32_t b, uint64_t base,
+                                            uint64_t min_d, uint32_t lane) {
+    using U = typename std::conditional<sizeof(T) == 8, unsigned long long, unsigned int>::type;
+    const uint32_t mask = (1u << b) - 1u;
+    const bool al32 = (reinterpret_cast<uintptr_t>(dst) & 31) == 0;
+    uint32_t carry = 0;                                    // differences of the steps before
+#pragma unroll 2
+    for (uint32_t j = 4 * lane; j - 4 * lane < mk; j += 128) {
+        uint32_t u[4];
+        delta_diffs<W>(wsm, j * b, b, mask, u);
+        if (j == 0) u[0] = 0;                              // u_0 of the block counts as 0
+        // values past the block (mk < 1024) take whatever the buffer holds after the payload: nothing is stored for them
+        u[1] += u[0];
+        u[2] += u[1];
+        u[3] += u[2];
+        const uint32_t incl = warp_incl_sum<uint32_t>(u[3], lane);
+        const uint32_t before = carry + incl - u[3];
+        carry += __shfl_sync(0xFFFFFFFFu, incl, 31);
+        T v[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if constexpr (OFF32) v[k] = (T)((U)base + ((j + k) * (uint32_t)min_d + (before + u[k])));
+            else v[k] = (T)((U)base + (U)(j + k) * (U)min_d + (U)(before + u[k]));
+        }
+        if (j + 4 <= mk) {
+            store_vec<T, 4>(dst + j, v, al32);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (j + k < mk) dst[j + k] = v[k];
+        }
+    }
+}
+
+template <class T, int W>
+__device__ __forceinline__ void delta_block_of(T* dst, const uint32_t* wsm, uint32_t mk, uint32_t b, uint64_t base,
+                                               uint64_t min_d, uint32_t lane) {
+    // min_d < 2^21: 1024 * (min_d + 2^b) < 2^32; 32-bit values need 32 bits anyway
+    if (sizeof(T) == 4 || min_d < (1u << 21)) delta_block<T, W, true>(dst, wsm, mk, b, base, min_d, lane);
+    else delta_block<T, W, false>(dst, wsm, mk, b, base, min_d, lane);
+}
+
+// Out of line, these rare blocks do not add to the registers of the common
+// path.  They keep 16-byte stores: in an out-of-line function a 256-bit store
+// from inline PTX wrote only part of its data (seen on GB300; the same store
+// inlined is exact).
 template <class T>
 __device__ __noinline__ void delta_block_wide(T* dst, const uint32_t* wsm, uint32_t mk, uint32_t b, uint64_t base,
                                               uint64_t min_d, uint32_t lane) {
-    delta_block_lanes<T, true, false>(dst, wsm, mk, b, base, min_d, lane, nullptr);
+    delta_block_lanes<T>(dst, wsm, mk, b, base, min_d, lane);
 }
 
 // Blocks of rows [r0, r0 + nrows) (r0 a multiple of 1024, at most 32 blocks).
@@ -585,8 +545,9 @@ __device__ void delta_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32
         if ((ok_mask >> i) & 1) {
             T* dst = reinterpret_cast<T*>(c.dst) + r0 + i * zf::kDeltaBlock;
             const uint32_t* buf = wsm + (i & 1) * sb;
-            uint4* xb = reinterpret_cast<uint4*>(wsm + 2 * sb);
-            if (b <= 21) delta_block_lanes<T, false, true>(dst, buf, mk, b, base, md, lane, xb);
+            if (b <= 8) delta_block_of<T, 1>(dst, buf, mk, b, base, md, lane);
+            else if (b <= 16) delta_block_of<T, 2>(dst, buf, mk, b, base, md, lane);
+            else if (b <= 21) delta_block_of<T, 4>(dst, buf, mk, b, base, md, lane);
             else delta_block_wide<T>(dst, buf, mk, b, base, md, lane);
         }
         __syncwarp();
@@ -822,8 +783,7 @@ constexpr uint32_t kStrWin = 16u * zf::kStrTokenMax + 32u;    // 16 tokens of at
 // the widest bit width of the chunks it decodes (two staging buffers).
 __host__ __device__ inline uint32_t warp_smem(int scheme, uint32_t value_bytes, uint32_t bmax) {
     switch (scheme) {
-    case ZF_FOR_BP: case ZF_DICT_BP: case ZF_FLOAT2INT: return 2 * stage_bytes_for(bmax);
-    case ZF_DELTA_BP: return 2 * stage_bytes_for(bmax) + 4096;   // + the store transpose buffer
+    case ZF_FOR_BP: case ZF_DICT_BP: case ZF_FLOAT2INT: case ZF_DELTA_BP: return 2 * stage_bytes_for(bmax);
     case ZF_RLE: return 128 + kRleStages * rle_buf_bytes(value_bytes);   // row bitmask + staging buffers
     case ZF_STRDICT: return kStrCodeBuf + kStrWin;                      // one tile of codes + the output window
     }
