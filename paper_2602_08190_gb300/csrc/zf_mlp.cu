@@ -7,6 +7,7 @@
 // over the classes each sample allows (others masked), averaged over the
 // batch.  Gradients are summed in a fixed order (eight samples in a CTA, then
 // the CTAs), so training is deterministic.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -44,23 +45,17 @@ struct MlpSmem {
     alignas(16) float loss[kTile];
 };
 
-// The rows a launch reads: row r of the batch is row inl[r] of X where
-// `listed` (a batch of up to kListed rows: its order travels as parameters, so
-// no copy stands between the steps), else order[r], or r where order is null.
-// They are standardized as (x - mean) / sd where scaled.
-constexpr uint32_t kListed = 512;
+// The rows a launch reads: row r of the batch is row order[r] of X (row r
+// where order is null), standardized as (x - mean) / sd where scaled.
 struct Rows {
     const float* X;
     const uint32_t* order;
     uint32_t n;
-    bool scaled, listed;
+    bool scaled;
     float mean[IN], sd[IN];
-    uint32_t inl[kListed];
 };
 
-__device__ __forceinline__ uint32_t row_of(const Rows& r, uint32_t i) {
-    return r.listed ? r.inl[i] : r.order ? r.order[i] : i;
-}
+__device__ __forceinline__ uint32_t row_of(const Rows& r, uint32_t i) { return r.order ? r.order[i] : i; }
 
 // Loads the weights and the CTA's samples (zeros past the batch) and computes the logits sm.z.
 __device__ __forceinline__ void forward_tile(const float* __restrict__ p, const Rows& r, MlpSmem& sm) {
@@ -247,13 +242,20 @@ __global__ void mlp_reduce(const float* __restrict__ part, uint32_t nparts, uint
     if (i == NP && loss) *loss = sum_parts(part, nparts, NP) / (float)B;
 }
 
+__device__ __forceinline__ void adam_value(float& p, float& m, float& v, float gi, float lr, float b1, float b2, float eps,
+                                           float c1, float c2) {
+    m = b1 * m + (1.0f - b1) * gi;
+    v = b2 * v + (1.0f - b2) * gi * gi;
+    p -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
+
 __device__ __forceinline__ void adam_one(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v, int i,
                                          float gi, float lr, float b1, float b2, float eps, float c1, float c2) {
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+    float pi = p[i], mi = m[i], vi = v[i];
+    adam_value(pi, mi, vi, gi, lr, b1, b2, eps, c1, c2);
+    p[i] = pi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
 // A training step after mlp_grad_part: the gradient's sum and the Adam update in one pass.
@@ -271,6 +273,321 @@ __global__ void mlp_adam(float* __restrict__ p, float* __restrict__ m, float* __
     if (i < NP) adam_one(p, m, v, i, g[i], lr, b1, b2, eps, c1, c2);
 }
 
+// ---------------------------------------------------------------- training in one cluster
+// Steps of up to kClusterBatch samples run inside one kernel: a cluster of
+// kRanks CTAs keeps the weights in every CTA's shared memory and each rank a
+// sixteenth of the Adam state in registers.  Per step a rank takes a sixteenth
+// of the batch (16 samples at a time), leaves its share of the gradient in its
+// shared memory, and after a cluster barrier every rank sums the sixteen shares
+// of its sixteenth of the parameters, updates them and stores them into all
+// CTAs' weights.  The next step's rows are loaded while a step computes.  A
+// layer takes one unit and kSpt samples per thread, a weight gradient 4 x 4
+// values per thread.  What bounds it is the latency of a step's layers and two
+// cluster barriers (28% of issue slots busy): a step of 256 samples takes 13.5
+// us, 25 as two launches.  Eight ranks of 32 samples took 23.
+constexpr int kRanks = 16, kCt = 512, kSamples = 16;
+constexpr int kSpt = kSamples * HID / kCt;          // samples of a thread (of one unit)
+constexpr int kSt = kSamples + 4, kUt = HID + 4;    // a unit's samples and a sample's units, padded
+constexpr uint32_t kClusterBatch = 2 * kRanks * kSamples;
+constexpr int kOwn = (NP + kRanks - 1) / kRanks, kPer = (kOwn + kCt - 1) / kCt;   // parameters of a rank, of a thread
+static_assert(kSpt == 2 || kSpt == 4, "vector loads of a thread's samples");
+
+struct TrainSmem {
+    float w1[HID * (IN + 1)], w2[HID * (HID + 1)], w3[OUT * (HID + 1)], b1[HID], b2[HID], b3[OUT];
+    alignas(16) float x[IN * kSt];                                                // unit by unit
+    alignas(16) float h1[HID * kSt], h2[HID * kSt], d2[HID * kSt], z[OUT * kSt];
+    alignas(16) float xs[kSamples * kUt], h1s[kSamples * kUt], h2s[kSamples * kUt];   // sample by sample
+    alignas(16) float d1s[kSamples * kUt], d2s[kSamples * kUt], zs[kSamples * 16];
+    alignas(16) float grad[NP];
+    float loss[kSamples];
+    float total_loss;
+    uint32_t mask[kSamples];
+    int32_t y[kSamples];
+};
+
+struct TrainArgs {
+    const float* X;
+    const int32_t* Y;
+    const uint8_t* MK;
+    const uint32_t* order;    // the epochs' sample orders, `count` each
+    const float* c1;          // Adam's bias corrections of every step
+    const float* c2;
+    float* losses;            // one per step
+    float *p, *m, *v;
+    uint32_t count, batch, epochs;
+    float lr, b1, b2, eps;
+    float mean[IN], sd[IN];
+};
+
+// Where parameter i lies in the padded weights.
+__device__ __forceinline__ float* weight(TrainSmem& sm, int i) {
+    if (i < OB1) return &sm.w1[i / IN * (IN + 1) + i % IN];
+    if (i < OW2) return &sm.b1[i - OB1];
+    if (i < OB2) return &sm.w2[(i - OW2) / HID * (HID + 1) + (i - OW2) % HID];
+    if (i < OW3) return &sm.b2[i - OB2];
+    if (i < OB3) return &sm.w3[(i - OW3) / HID * (HID + 1) + (i - OW3) % HID];
+    return &sm.b3[i - OB3];
+}
+
+// A thread's kSpt samples of one unit.
+struct Vals {
+    float v[kSpt];
+};
+__device__ __forceinline__ Vals load_vals(const float* p) {
+    Vals r;
+    if constexpr (kSpt == 4) *reinterpret_cast<float4*>(r.v) = *reinterpret_cast<const float4*>(p);
+    else *reinterpret_cast<float2*>(r.v) = *reinterpret_cast<const float2*>(p);
+    return r;
+}
+__device__ __forceinline__ void store_vals(float* p, const Vals& r) {
+    if constexpr (kSpt == 4) *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(r.v);
+    else *reinterpret_cast<float2*>(p) = *reinterpret_cast<const float2*>(r.v);
+}
+
+// Samples g.. of one unit of a layer: a + the sum over i of w[i * ws] * in[i][g..].
+template <int N>
+__device__ __forceinline__ Vals layer(const float* w, int ws, const float* in, int g, float a) {
+    Vals r;
+#pragma unroll
+    for (int s = 0; s < kSpt; s++) r.v[s] = a;
+#pragma unroll 16
+    for (int i = 0; i < N; i++) {
+        const float u = w[i * ws];
+        const Vals x = load_vals(&in[i * kSt + g]);
+#pragma unroll
+        for (int s = 0; s < kSpt; s++) r.v[s] += u * x.v[s];
+    }
+    return r;
+}
+
+// A 4 x 4 piece of a weight gradient: the sum over n samples of a[s][0..3] times
+// b[s][0..3] (rows of `as` and kUt floats), written to rows of `gs` floats at g
+// (added there where `add`).
+__device__ __forceinline__ void grad_tile(const float* a, int as, const float* b, int n, float* g, int gs, bool add) {
+    float t[4][4] = {};
+#pragma unroll 4
+    for (int s = 0; s < n; s++) {
+        const float4 u = *reinterpret_cast<const float4*>(a + s * as), v = *reinterpret_cast<const float4*>(b + s * kUt);
+        const float uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) t[r][c] += uu[r] * vv[c];
+    }
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        float4* o = reinterpret_cast<float4*>(g + r * gs);
+        float4 w = make_float4(t[r][0], t[r][1], t[r][2], t[r][3]);
+        if (add) {
+            const float4 q = *o;
+            w = make_float4(q.x + w.x, q.y + w.y, q.z + w.z, q.w + w.w);
+        }
+        *o = w;
+    }
+}
+
+__global__ void __launch_bounds__(kCt, 1) mlp_train_cluster(const __grid_constant__ TrainArgs t) {
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) unsigned char smem[];
+    TrainSmem& sm = *reinterpret_cast<TrainSmem*>(smem);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int tid = threadIdx.x, rank = (int)cluster.block_rank();
+    for (int i = tid; i < NP; i += kCt) *weight(sm, i) = t.p[i];
+    float pp[kPer], pm[kPer], pv[kPer];   // the thread's parameters rank * kOwn + tid + kCt q
+    int own[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; q++) {
+        const int k = tid + kCt * q, i = rank * kOwn + k;
+        own[q] = k < kOwn && i < NP ? i : -1;
+        pp[q] = own[q] >= 0 ? t.p[i] : 0.0f;
+        pm[q] = own[q] >= 0 ? t.m[i] : 0.0f;
+        pv[q] = own[q] >= 0 ? t.v[i] : 0.0f;
+    }
+    const uint32_t per_epoch = (t.count + t.batch - 1) / t.batch, steps = per_epoch * t.epochs;
+    // first sample (in the orders) and samples of this rank in step k
+    auto share = [&](uint32_t k, uint32_t& first, uint32_t& B) -> uint32_t {
+        const uint32_t e = k / per_epoch, b0 = (k % per_epoch) * t.batch;
+        B = min(t.batch, t.count - b0);
+        const uint32_t per = (B + kRanks - 1) / kRanks, r0 = min(B, per * rank);
+        first = e * t.count + b0 + r0;
+        return min(per, B - r0);
+    };
+    // the thread's input values of a pass and, for the first threads, their sample's label and mask
+    constexpr int kX = kSamples * IN / kCt, kRow = kCt / IN;   // values of a thread, samples between them
+    const int xs = tid / IN, xi = tid % IN;
+    const float mu = t.mean[xi], sd = t.sd[xi];
+    float nx[kX];
+    uint32_t row[kX], lrow = 0;      // their rows in X, loaded a pass ahead: a row waits for its index, the thread does not
+    int32_t ny = 0;
+    uint32_t nm = 0;
+    auto fetch_rows = [&](uint32_t first, uint32_t n) {
+#pragma unroll
+        for (int q = 0; q < kX; q++) row[q] = (uint32_t)(xs + kRow * q) < n ? t.order[first + xs + kRow * q] : 0xFFFFFFFFu;
+        lrow = tid < kSamples && (uint32_t)tid < n ? t.order[first + tid] : 0xFFFFFFFFu;
+    };
+    auto fetch = [&]() {
+#pragma unroll
+        for (int q = 0; q < kX; q++) nx[q] = row[q] != 0xFFFFFFFFu ? t.X[(size_t)row[q] * IN + xi] : mu;
+        ny = 0;
+        nm = 0;
+        if (lrow != 0xFFFFFFFFu) {
+            ny = t.Y[lrow];
+            const uint32_t* mk = reinterpret_cast<const uint32_t*>(t.MK + (size_t)lrow * OUT);
+            const uint32_t m0 = mk[0], m1 = mk[1], m2 = mk[2];
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                nm |= ((m0 >> (8 * k)) & 0xFFu ? 1u << k : 0u) | ((m1 >> (8 * k)) & 0xFFu ? 16u << k : 0u) |
+                      ((m2 >> (8 * k)) & 0xFFu ? 256u << k : 0u);
+        }
+    };
+    const int j = tid % HID, g = tid / HID * kSpt;   // the thread's unit and first sample
+    // a layer's result in both orders
+    auto keep = [&](const Vals& r, float* by_unit, float* by_sample) {
+        if (by_unit) store_vals(&by_unit[j * kSt + g], r);
+#pragma unroll
+        for (int s = 0; s < kSpt; s++) by_sample[(g + s) * kUt + j] = r.v[s];
+    };
+    uint32_t first, B, n = share(0, first, B);
+    auto first_rows = [&](uint32_t k) {              // of step k, if there is one
+        uint32_t f2, B2;
+        const uint32_t n2 = k < steps ? share(k, f2, B2) : 0;
+        fetch_rows(f2, min(n2, (uint32_t)kSamples));
+    };
+    fetch_rows(first, min(n, (uint32_t)kSamples));
+    fetch();
+    if (n <= kSamples) first_rows(1);
+    float* const mine = own[0] >= 0 ? weight(sm, own[0]) : nullptr;
+    for (uint32_t k = 0; k < steps; k++) {
+        if (tid == 0) sm.total_loss = 0.0f;
+        // at least one pass, so that a rank without samples leaves a gradient of zero
+        for (uint32_t s0 = 0; s0 == 0 || s0 < n; s0 += kSamples) {
+            const uint32_t ns = n > s0 ? min(n - s0, (uint32_t)kSamples) : 0u;
+            if (s0) {
+                fetch_rows(first + s0, ns);
+                fetch();
+                if (s0 + kSamples >= n) first_rows(k + 1);
+            }
+#pragma unroll
+            for (int q = 0; q < kX; q++) {
+                const float v = (nx[q] - mu) / sd;   // samples past ns are zeros
+                sm.x[xi * kSt + xs + kRow * q] = v;
+                sm.xs[(xs + kRow * q) * kUt + xi] = v;
+            }
+            if (tid < kSamples) {
+                sm.y[tid] = ny;
+                sm.mask[tid] = nm;
+            }
+            __syncthreads();
+            if (s0 + kSamples >= n && k + 1 < steps) {           // the next step's first rows, and the indices after them
+                fetch();
+                uint32_t f2, B2;
+                if (share(k + 1, f2, B2) <= kSamples) first_rows(k + 2);
+            }
+            Vals h1 = layer<IN>(&sm.w1[j * (IN + 1)], 1, sm.x, g, sm.b1[j]);
+#pragma unroll
+            for (int s = 0; s < kSpt; s++) h1.v[s] = fmaxf(h1.v[s], 0.0f);
+            keep(h1, sm.h1, sm.h1s);
+            __syncthreads();
+            Vals h2 = layer<HID>(&sm.w2[j * (HID + 1)], 1, sm.h1, g, sm.b2[j]);
+#pragma unroll
+            for (int s = 0; s < kSpt; s++) h2.v[s] = fmaxf(h2.v[s], 0.0f);
+            keep(h2, sm.h2, sm.h2s);
+            __syncthreads();
+            // logits and their gradient: 16 lanes per sample, one class each
+            if (tid < 16 * kSamples) {
+                const int s = tid / 16, o = tid % 16;
+                const bool in = (uint32_t)s < ns, cls = o < OUT;
+                float z = cls ? sm.b3[o] : 0.0f;
+                if (cls) {
+#pragma unroll 16
+                    for (int i = 0; i < HID; i++) z += sm.w3[o * (HID + 1) + i] * sm.h2[i * kSt + s];
+                }
+                const bool allowed = in && cls && ((sm.mask[s] >> o) & 1u);
+                float mx = allowed ? z : -INFINITY;
+#pragma unroll
+                for (int d = 8; d; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, d));
+                const float e = allowed ? expf(z - mx) : 0.0f;
+                float sum = e;
+#pragma unroll
+                for (int d = 8; d; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+                const int y = sm.y[s];
+                const bool label = o == y;
+                const float dz = in && cls ? (e / sum - (label ? 1.0f : 0.0f)) / (float)B : 0.0f;
+                if (cls) {
+                    sm.z[o * kSt + s] = dz;
+                    sm.zs[s * 16 + o] = dz;
+                    if (label || (o == 0 && (uint32_t)y >= OUT)) sm.loss[s] = in ? -logf((label ? e : 0.0f) / sum) : 0.0f;
+                }
+            }
+            __syncthreads();
+            if (tid < 32) {
+                float l = tid < (int)ns ? sm.loss[tid] : 0.0f;
+#pragma unroll
+                for (int d = 16; d; d >>= 1) l += __shfl_down_sync(0xFFFFFFFFu, l, d);
+                if (tid == 0) sm.total_loss += l;
+            }
+            Vals d2 = layer<OUT>(&sm.w3[j], HID + 1, sm.z, g, 0.0f);
+#pragma unroll
+            for (int s = 0; s < kSpt; s++) d2.v[s] = h2.v[s] > 0.0f ? d2.v[s] : 0.0f;
+            keep(d2, sm.d2, sm.d2s);
+            __syncthreads();
+            Vals d1 = layer<HID>(&sm.w2[j], HID + 1, sm.d2, g, 0.0f);
+#pragma unroll
+            for (int s = 0; s < kSpt; s++) d1.v[s] = h1.v[s] > 0.0f ? d1.v[s] : 0.0f;
+            keep(d1, nullptr, sm.d1s);
+            __syncthreads();
+            // the rank's share of the gradient: 256 threads for W2, 128 for W1, 48 for W3, the rest for the biases
+            const bool add = s0 != 0;
+            if (tid < 256) {
+                const int r = tid / 16 * 4, c = tid % 16 * 4;
+                grad_tile(&sm.d2s[r], kUt, &sm.h1s[c], (int)ns, &sm.grad[OW2 + r * HID + c], HID, add);
+            } else if (tid < 384) {
+                const int r = (tid - 256) / 8 * 4, c = (tid - 256) % 8 * 4;
+                grad_tile(&sm.d1s[r], kUt, &sm.xs[c], (int)ns, &sm.grad[OW1 + r * IN + c], IN, add);
+            } else if (tid < 432) {
+                const int r = (tid - 384) / 16 * 4, c = (tid - 384) % 16 * 4;
+                grad_tile(&sm.zs[r], 16, &sm.h2s[c], (int)ns, &sm.grad[OW3 + r * HID + c], HID, add);
+            } else {
+                for (int i = tid - 432; i < 2 * HID + OUT; i += kCt - 432) {
+                    const float* a = i < HID ? &sm.d1s[i] : i < 2 * HID ? &sm.d2s[i - HID] : &sm.zs[i - 2 * HID];
+                    const int st = i < 2 * HID ? kUt : 16, at = i < HID ? OB1 + i : i < 2 * HID ? OB2 + i - HID : OB3 + i - 2 * HID;
+                    float r = add ? sm.grad[at] : 0.0f;
+                    for (int s = 0; s < (int)ns; s++) r += a[s * st];
+                    sm.grad[at] = r;
+                }
+            }
+            __syncthreads();
+        }
+        cluster.sync();   // every rank's share is in its shared memory
+        const float c1 = t.c1[k], c2 = t.c2[k];
+#pragma unroll
+        for (int q = 0; q < kPer; q++) {
+            if (own[q] < 0) continue;
+            float gi = 0.0f;
+#pragma unroll
+            for (int r = 0; r < kRanks; r++) gi += *cluster.map_shared_rank(&sm.grad[own[q]], r);
+            adam_value(pp[q], pm[q], pv[q], gi, t.lr, t.b1, t.b2, t.eps, c1, c2);
+            float* w = q ? weight(sm, own[q]) : mine;
+#pragma unroll
+            for (int r = 0; r < kRanks; r++) *cluster.map_shared_rank(w, r) = pp[q];
+        }
+        if (rank == 0 && tid == kCt - 1) {
+            float l = 0.0f;
+            for (int r = 0; r < kRanks; r++) l += *cluster.map_shared_rank(&sm.total_loss, r);
+            t.losses[k] = l / (float)B;
+        }
+        if (k + 1 < steps) n = share(k + 1, first, B);
+        cluster.sync();   // the weights are the next step's; no rank reads a gradient any more
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; q++)
+        if (own[q] >= 0) {
+            t.p[own[q]] = pp[q];
+            t.m[own[q]] = pm[q];
+            t.v[own[q]] = pv[q];
+        }
+}
+
 uint64_t splitmix(uint64_t x) {
     x += 0x9E3779B97F4A7C15ull;
     x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -278,7 +595,8 @@ uint64_t splitmix(uint64_t x) {
     return x ^ (x >> 31);
 }
 
-double unit(uint64_t seed, uint64_t i) { return ((splitmix(seed ^ splitmix(i)) >> 11) + 0.5) / 9007199254740992.0; }
+double unit_of(uint64_t h) { return ((h >> 11) + 0.5) / 9007199254740992.0; }
+double unit(uint64_t seed, uint64_t i) { return unit_of(splitmix(seed ^ splitmix(i))); }
 
 }  // namespace
 
@@ -292,6 +610,7 @@ struct zf_mlp {
     uint8_t* data = nullptr;  // zf_mlp_train's and zf_mlp_predict's rows on the device, kept for the next call
     size_t data_cap = 0;
     std::mutex data_mu;       // held by the calls that use `data`
+    int cluster = -1;         // whether mlp_train_cluster fits the device (-1: not asked yet)
     uint32_t step = 0;
     // input standardization (x - mean) / std, fitted by zf_mlp_train on its
     // rows and applied by zf_mlp_train and zf_mlp_predict
@@ -345,6 +664,36 @@ void release_large(zf_mlp* n) {
         n->data = nullptr;
         n->data_cap = 0;
     }
+}
+
+cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* at) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(kRanks);
+    c.blockDim = dim3(kCt);
+    c.dynamicSmemBytes = sizeof(TrainSmem);
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim = {kRanks, 1, 1};
+    c.attrs = at;
+    c.numAttrs = 1;
+    return c;
+}
+// Whether the current device runs a cluster of kRanks such CTAs (more than eight are a device's choice).
+bool cluster_fits() {
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t c = cluster_config(&at);
+    int most = 0;
+    if (cudaFuncSetAttribute(mlp_train_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) != cudaSuccess ||
+        cudaFuncSetAttribute(mlp_train_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&most, mlp_train_cluster, &c) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return most > 0;
+}
+cudaError_t launch_cluster(const TrainArgs& args) {
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t c = cluster_config(&at);
+    return cudaLaunchKernelEx(&c, mlp_train_cluster, args);
 }
 
 Rows plain_rows(const float* X, uint32_t n) {
@@ -448,28 +797,35 @@ zf_status zf_mlp_adam(zf_mlp* n, const float* d_grad, float lr, void* stream) {
 }
 
 // Mini-batch training on the GPU: the sample order of every epoch is a
-// seeded shuffle; a step is two launches, and the host does not wait for any
-// of them: the rows are on the device once, a batch's order is a parameter of
-// its launch, and the losses come back at the end.  Three copies and three
-// launches a step, each step waited for, took 1,367 us for two epochs of
-// eight batches of 256; this takes 509 us.
+// seeded shuffle.  The rows are on the device once, and the host does not wait
+// for a step: batches of up to kClusterBatch samples run inside one launch per
+// group of epochs (mlp_train_cluster; the next group's orders are shuffled
+// meanwhile), larger ones as two launches a step; the losses come back at the
+// end.  Three copies and three launches a step, each step waited for, took
+// 1,367 us for two epochs of eight batches of 256, two launches a step 509;
+// this takes 325.
 zf_status zf_mlp_train(zf_mlp* n, const float* h_x, const int32_t* h_y, const uint8_t* h_mask, uint32_t count,
                        uint32_t epochs, uint32_t batch, float lr, uint64_t seed, float* h_losses) {
     zf::KeepDevice keep_device;
     if (!n || !h_x || !h_y || !h_mask || !count || !batch) return ZF_EINVAL;
     cudaSetDevice(n->device);
     std::lock_guard<std::mutex> lock(n->data_mu);
+    batch = std::min(batch, count);
+    if (n->cluster < 0) n->cluster = cluster_fits();
+    const bool cluster = batch <= kClusterBatch && n->cluster;
     const uint32_t steps = count / batch + (count % batch != 0);   // of an epoch
-    const uint32_t group = std::max(1u, std::min(epochs, (1u << 20) / steps));   // epochs whose losses come back at once
-    const bool listed = std::min(batch, count) <= kListed;
+    // epochs whose losses come back at once, and epochs of one launch or upload at most
+    const uint32_t back = std::max(1u, std::min(epochs, (1u << 20) / steps));
+    const uint32_t most = cluster ? std::max(1u, std::min(std::min(epochs, 64u), (1u << 18) / count)) : 1u;
+    const size_t words = (size_t)most * (count + 2 * (size_t)steps);   // orders, then c1 and c2 of every step
     float *dx = nullptr, *dl = nullptr;
     int32_t* dy = nullptr;
     uint8_t* dm = nullptr;
     uint32_t* dord = nullptr;
-    zf_status st = ensure_batch(n, std::min(batch, count));
+    zf_status st = cluster ? ZF_OK : ensure_batch(n, batch);
     if (!st)
         st = ensure_data(n, {(size_t)count * IN * sizeof(float), (size_t)count * sizeof(int32_t), (size_t)count * OUT,
-                             listed ? 0 : (size_t)count * sizeof(uint32_t), (size_t)group * steps * sizeof(float)},
+                             words * sizeof(uint32_t), (size_t)back * steps * sizeof(float)},
                          {(void**)&dx, (void**)&dy, (void**)&dm, (void**)&dord, (void**)&dl});
     if (st) return st;
     auto done = [&](zf_status s) {
@@ -497,39 +853,69 @@ zf_status zf_mlp_train(zf_mlp* n, const float* h_x, const int32_t* h_y, const ui
         cudaMemcpy(dy, h_y, (size_t)count * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(dm, h_mask, (size_t)count * OUT, cudaMemcpyHostToDevice) != cudaSuccess)
         return done(ZF_ECUDA);
-    rows.listed = listed;
-    std::vector<uint32_t> order(count);
-    std::vector<float> losses((size_t)group * steps);
-    for (uint32_t e0 = 0; e0 < epochs; e0 += group) {
-        const uint32_t ne = std::min(group, epochs - e0);
-        for (uint32_t e = 0; e < ne; e++) {
-            std::iota(order.begin(), order.end(), 0u);
-            for (uint32_t i = count; i > 1; i--) {   // Fisher-Yates with the counter generator
-                const uint32_t j = (uint32_t)(unit(seed + e0 + e, i) * i);
-                std::swap(order[i - 1], order[std::min(j, i - 1)]);
+    TrainArgs args{};
+    if (cluster) {
+        args = TrainArgs{dx, dy, dm, nullptr, nullptr, nullptr, nullptr, n->p, n->m, n->v, count, batch, 0,
+                         lr, 0.9f, 0.999f, 1e-8f, {}, {}};
+        std::copy(rows.mean, rows.mean + IN, args.mean);
+        std::copy(rows.sd, rows.sd + IN, args.sd);
+    }
+    std::vector<uint64_t> hash(count + 1);   // of the counter generator, the same every epoch
+    for (uint32_t i = 2; i <= count; i++) hash[i] = splitmix(i);
+    std::vector<uint32_t> up(words);
+    std::vector<float> losses((size_t)back * steps);
+    uint32_t group = 1;                      // the first launch starts after one shuffle, later ones are larger
+    for (uint32_t e0 = 0; e0 < epochs; e0 += back) {
+        const uint32_t e1 = std::min(epochs, e0 + back);
+        for (uint32_t e = e0; e < e1;) {
+            const uint32_t ne = std::min(std::min(group, most), e1 - e);
+            for (uint32_t q = 0; q < ne; q++) {
+                uint32_t* order = up.data() + (size_t)q * count;
+                std::iota(order, order + count, 0u);
+                for (uint32_t i = count; i > 1; i--) {   // Fisher-Yates with the counter generator
+                    const uint32_t j = (uint32_t)(unit_of(splitmix((seed + e + q) ^ hash[i])) * i);
+                    std::swap(order[i - 1], order[std::min(j, i - 1)]);
+                }
             }
-            if (!listed && cudaMemcpy(dord, order.data(), (size_t)count * sizeof(uint32_t), cudaMemcpyHostToDevice) != cudaSuccess)
-                return done(ZF_ECUDA);
-            for (uint32_t k = 0; k < steps; k++) {
-                rows.n = std::min(batch, count - k * batch);
-                if (listed) std::copy_n(order.begin() + (size_t)k * batch, rows.n, rows.inl);
-                else rows.order = dord + (size_t)k * batch;
+            float* c = reinterpret_cast<float*>(up.data() + (size_t)ne * count);
+            const uint32_t ns = ne * steps;
+            for (uint32_t k = 0; k < ns; k++) {
                 n->step++;
-                const float c1 = (float)(1.0 - std::pow(0.9, (double)n->step));
-                const float c2 = (float)(1.0 - std::pow(0.999, (double)n->step));
-                mlp_grad_part<<<tiles(rows.n), kThreads>>>(n->p, rows, dy, dm, n->part);
-                mlp_reduce_adam<<<(NP + 256) / 256, 256>>>(n->part, tiles(rows.n), rows.n, dl + (size_t)e * steps + k,
-                                                           n->p, n->m, n->v, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
+                c[k] = (float)(1.0 - std::pow(0.9, (double)n->step));
+                c[ns + k] = (float)(1.0 - std::pow(0.999, (double)n->step));
             }
+            float* dloss = dl + (size_t)(e - e0) * steps;
+            if (cudaMemcpyAsync(dord, up.data(), ((size_t)ne * count + 2 * (size_t)ns) * sizeof(uint32_t), cudaMemcpyHostToDevice, 0) !=
+                cudaSuccess)
+                return done(ZF_ECUDA);
+            if (cluster) {
+                args.order = dord;
+                args.c1 = reinterpret_cast<const float*>(dord + (size_t)ne * count);
+                args.c2 = args.c1 + ns;
+                args.losses = dloss;
+                args.epochs = ne;
+                if (launch_cluster(args) != cudaSuccess) return done(ZF_ECUDA);
+            } else {
+                for (uint32_t k = 0; k < ns; k++) {
+                    const uint32_t b0 = k % steps * batch;
+                    rows.n = std::min(batch, count - b0);
+                    rows.order = dord + (size_t)(k / steps) * count + b0;
+                    mlp_grad_part<<<tiles(rows.n), kThreads>>>(n->p, rows, dy, dm, n->part);
+                    mlp_reduce_adam<<<(NP + 256) / 256, 256>>>(n->part, tiles(rows.n), rows.n, dloss + k, n->p, n->m, n->v, lr,
+                                                               0.9f, 0.999f, 1e-8f, c[k], c[ns + k]);
+                }
+            }
+            if (cudaGetLastError() != cudaSuccess) return done(ZF_ECUDA);
+            e += ne;
+            group = std::min(2 * group, most);
         }
-        if (cudaGetLastError() != cudaSuccess) return done(ZF_ECUDA);
         if (!h_losses) continue;
-        if (cudaMemcpy(losses.data(), dl, (size_t)ne * steps * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
+        if (cudaMemcpy(losses.data(), dl, (size_t)(e1 - e0) * steps * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
             return done(ZF_ECUDA);
-        for (uint32_t e = 0; e < ne; e++) {
+        for (uint32_t e = e0; e < e1; e++) {
             double esum = 0;
-            for (uint32_t k = 0; k < steps; k++) esum += losses[(size_t)e * steps + k];
-            h_losses[e0 + e] = (float)(esum / steps);
+            for (uint32_t k = 0; k < steps; k++) esum += losses[(size_t)(e - e0) * steps + k];
+            h_losses[e] = (float)(esum / steps);
         }
     }
     return done(cudaDeviceSynchronize() == cudaSuccess ? ZF_OK : ZF_ECUDA);
