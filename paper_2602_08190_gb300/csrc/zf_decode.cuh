@@ -5,8 +5,9 @@
 
 namespace zfd {
 
-// Decode rows [r0, r0 + nrows) of a chunk (string dictionary: tokens) by one warp.
-template <int SCHEME, int DT>
+// Decode rows [r0, r0 + nrows) of a chunk (string dictionary: tokens) by one
+// warp.  MIXED: the kernel decodes every scheme.
+template <int SCHEME, int DT, bool MIXED>
 __device__ __forceinline__ void decode_one(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t nrows,
                                            uint32_t* wsm, uint32_t* err) {
     if constexpr (DT == ZF_I32 || DT == ZF_I64) {
@@ -16,7 +17,7 @@ __device__ __forceinline__ void decode_one(const ZfDevChunk& c, const Hdr& h, ui
         else if constexpr (SCHEME == ZF_DELTA_BP)
             delta_job<T>(c, h, r0, nrows, wsm, err, c.bmax);
         else if constexpr (SCHEME == ZF_RLE)
-            rle_job<T>(c, h, r0, nrows, wsm, err);
+            rle_job<T, MIXED>(c, h, r0, nrows, wsm, err);
     } else if constexpr (DT == ZF_F64) {
         // doubles travel as their 64-bit patterns
         if constexpr (SCHEME == ZF_RAW || SCHEME == ZF_FLOAT2INT) fp_job<int64_t, SCHEME>(c, h, r0, nrows, wsm, err);

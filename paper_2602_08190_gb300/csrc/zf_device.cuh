@@ -20,7 +20,7 @@
 //               coalesced vector store per lane.
 //   rle_job     Group-Parallel: the tile's run lengths (the chunk's 1024-row
 //               directory names the first run) are scanned into start rows,
-//               four per lane and one warp shuffle scan per 128 runs (the
+//               four or eight per lane and one warp shuffle scan (the
 //               presum of Section 3.2); every run but the first sets its start
 //               row's bit in a 32-word bitmask, and a row's run is the number
 //               of set bits at or before it.  Each tile writes exactly 1024
@@ -143,17 +143,6 @@ __device__ __forceinline__ S warp_incl_sum(S x, uint32_t lane) {
     for (int d = 1; d < 32; d <<= 1) {
         S y = __shfl_up_sync(0xFFFFFFFFu, x, d);
         if (lane >= (uint32_t)d) x += y;
-    }
-    return x;
-}
-
-// Inclusive sum over the lanes of values <= cap, saturating at cap (cap <
-// 2^31, so no partial sum wraps).
-__device__ __forceinline__ uint32_t warp_incl_sum_sat(uint32_t x, uint32_t cap, uint32_t lane) {
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
-        if (lane >= (uint32_t)d) x = min(x + y, cap);
     }
     return x;
 }
@@ -558,77 +547,87 @@ __device__ void delta_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32
 }
 
 // ---------------------------------------------------------------- RLE (Group-Parallel)
+// Start bits of the runs whose lengths are entries [sft, sft + m) of lens_al,
+// PER entries per lane and step: the prefix sums give each run its start row in
+// the tile, and every run but the first (whose start is at or before row 0)
+// sets its bit.  A length counts as at most kLong rows, the first without the
+// `skip` rows before the tile: the lengths that decide anything are those that
+// end inside the tile, so no sum comes near 2^32 whatever the stream holds.
+// Returns whether a length is zero or longer than the chunk; `end` = the rows
+// covered from the tile's first row on, `last_start` = the last run's start.
+template <int PER>
+__device__ __forceinline__ bool rle_starts(const uint32_t* lens_al, uint32_t sft, uint32_t m, uint32_t skip, uint32_t nr,
+                                           uint32_t chunk_rows, uint32_t* bm, uint32_t lane, uint32_t& end,
+                                           uint32_t& last_start) {
+    constexpr uint32_t kLong = 2048;
+    const uint32_t n = sft + m;   // entries from the aligned start
+    bool bad = false;
+    end = 0;
+    uint32_t mine = 0;
+    for (uint32_t g = 0; g < n; g += 32 * PER) {
+        const uint32_t k0 = g + PER * lane;
+        uint32_t L[PER];
+#pragma unroll
+        for (int q = 0; q < PER / 4; q++) {
+            const uint4 x = k0 + 4 * q < n ? reinterpret_cast<const uint4*>(lens_al)[(k0 >> 2) + q] : make_uint4(0, 0, 0, 0);
+            L[4 * q] = x.x;
+            L[4 * q + 1] = x.y;
+            L[4 * q + 2] = x.z;
+            L[4 * q + 3] = x.w;
+        }
+        uint32_t sum = 0;
+#pragma unroll
+        for (int e = 0; e < PER; e++) {
+            const bool valid = k0 + e - sft < m;
+            bad |= valid && L[e] - 1u >= chunk_rows;
+            if (e < 4 && k0 + e == sft) {                      // the first run: entry 0..3 of lane 0
+                bad |= skip >= L[e];
+                L[e] -= min(skip, L[e]);
+            }
+            L[e] = valid ? min(L[e], kLong) : 0u;
+            sum += L[e];
+        }
+        const uint32_t incl = warp_incl_sum<uint32_t>(sum, lane);
+        uint32_t st = end + incl - sum;                        // start of entry k0
+        end += __shfl_sync(0xFFFFFFFFu, incl, 31);
+#pragma unroll
+        for (int e = 0; e < PER; e++) {
+            // starts 1 .. nr - 1: the first run's is 0, entries past the last start at nr or later
+            if (st - 1u < nr - 1u && k0 + e < n) atomicOr(&bm[st >> 5], 1u << (st & 31));
+            if (k0 + e + 1 == n) mine = st;
+            st += L[e];
+        }
+    }
+    last_start = __shfl_sync(0xFFFFFFFFu, mine, ((n - 1) % (32 * PER)) / PER);
+    return bad;
+}
+
 // Expansion of one 1024-row tile whose runs [rf, rf+m) have their lengths at
 // `lens_al` + sft, lens_al 16-byte aligned and sft = rf mod 4 (staged in shared
 // memory, or in global memory when the tile has more runs than a staging
 // buffer holds), and their values at `vals`.  `bm` is the warp's 32-word
 // bitmask of the tile's rows.
-template <class T>
+// TIGHT: four entries per lane and step only, for a kernel that decodes every
+// scheme and would spill registers with eight.
+// What bounds it: issue slots with short runs, DRAM from runs of 64 on.  64M
+// int32 rows in runs of mean 2, 4, 8 and 64: 152, 117, 78 and 70 us per
+// resident call; with saturating sums, four entries a step whatever the tile
+// and start bits merged per word in registers 181, 130, 83 and 73.
+template <class T, bool TIGHT>
 __device__ __forceinline__ void rle_rows(const ZfDevChunk& c, const Hdr& h, T* dst, const uint32_t* lens_al,
                                          uint32_t sft, const T* vals, uint32_t* bm, uint32_t m, uint32_t skip,
                                          uint32_t nr, bool last_tile, uint32_t next_skip, uint32_t lane,
                                          uint32_t* err) {
     bm[lane] = 0;
     __syncwarp();
-    // presum, 128 length entries per step: lane l reads entries 4l..4l+3 with
-    // one 16-byte load (entry sft is the tile's first run), one warp scan of
-    // the lanes' sums gives each run its start row relative to the first
-    // run's start, and every run but the first sets the bit of its start row.
-    // The tile's runs lie inside the chunk, so their lengths add up to at most
-    // its rows (<= 2^30); sums saturate at kCap = 2^30 + 1, which no valid
-    // tile reaches, so a stream whose lengths would wrap 32 bits is caught.
-    constexpr uint32_t kCap = (1u << 30) + 1u;
-    bool bad = false;
-    uint32_t end = 0;                 // rows covered so far, counted from the first run's start
-    uint32_t first_len = 0, my_last = 0;
-    const uint32_t n = sft + m;       // entries from the aligned start
-    for (uint32_t g = 0; g < n; g += 128) {
-        const uint32_t k0 = g + 4 * lane;
-        const uint4 q = k0 < n ? reinterpret_cast<const uint4*>(lens_al)[k0 >> 2] : make_uint4(0, 0, 0, 0);
-        uint32_t L[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int e = 0; e < 4; e++) {
-            const uint32_t k = k0 + e;
-            const bool valid = k >= sft && k < n;
-            if (!valid) L[e] = 0;
-            bad |= valid && (L[e] == 0 || L[e] > h.rows);
-        }
-        const uint32_t s4 = min(min(L[0] + L[1], kCap) + min(L[2] + L[3], kCap), kCap);
-        const uint32_t incl = warp_incl_sum_sat(s4, kCap, lane);
-        uint32_t st = end + incl - s4;  // start of entry k0
-        // the lane's start bits, ORed per bitmask word in registers first (its
-        // runs are consecutive, so their words are nondecreasing): one shared
-        // atomic per word the lane touches instead of one per run
-        uint32_t cw = 0xFFFFFFFFu, cbits = 0;
-#pragma unroll
-        for (int e = 0; e < 4; e++) {
-            const uint32_t k = k0 + e;
-            if (k > sft && k < n && st >= skip && st - skip < nr) {
-                const uint32_t r = st - skip;
-                if ((r >> 5) != cw) {
-                    if (cbits) atomicOr(&bm[cw], cbits);
-                    cw = r >> 5;
-                    cbits = 0;
-                }
-                cbits |= 1u << (r & 31);
-            }
-            if (k + 1 == n) my_last = st;
-            st += L[e];
-        }
-        if (cbits) atomicOr(&bm[cw], cbits);
-        if (g == 0) {
-            const uint32_t f0 = sft == 0 ? L[0] : sft == 1 ? L[1] : sft == 2 ? L[2] : L[3];
-            first_len = __shfl_sync(0xFFFFFFFFu, f0, 0);   // run 0: entry sft of lane 0
-        }
-        end = min(end + __shfl_sync(0xFFFFFFFFu, incl, 31), kCap);
-        if (end > h.rows) bad = true;
-    }
-    const uint32_t last_start = __shfl_sync(0xFFFFFFFFu, my_last, ((n - 1) & 127) >> 2);
-    // The runs cover exactly [0, nr): the first starts at or before row 0, the
-    // last ends at nr or continues into the next tile by the directory's amount.
-    bool ok = skip < first_len && end >= skip;
-    if (last_tile || next_skip == 0) ok &= end - skip == nr;
-    else ok &= last_start - skip + next_skip == nr && end - skip > nr;
+    uint32_t end, last_start;
+    bool bad;
+    if (TIGHT || sft + m <= 128) bad = rle_starts<4>(lens_al, sft, m, skip, nr, h.rows, bm, lane, end, last_start);
+    else bad = rle_starts<8>(lens_al, sft, m, skip, nr, h.rows, bm, lane, end, last_start);
+    // The runs cover exactly [0, nr): the last ends at nr or continues into the
+    // next tile by the directory's amount (a single run started `skip` rows before).
+    if (m == 1) last_start = 0u - skip;
+    const bool ok = last_tile || next_skip == 0 ? end == nr : last_start + next_skip == nr && end > nr;
     const bool any_bad = __any_sync(0xFFFFFFFFu, bad);
     if (lane == 0 && (!ok || any_bad)) report(err, ZF_ECORRUPT, c.chunk_id);
     __syncwarp();
@@ -685,11 +684,11 @@ __host__ __device__ inline uint32_t rle_buf_bytes(uint32_t value_bytes) {
 // Tiles of rows [r0, r0 + nrows) (r0 a multiple of 1024, at most 31 tiles).
 // Lane j holds the directory entry of tile j (and of the tile after the
 // last); the next tile's lengths and values are staged while a tile expands.
-template <class T>
+template <class T, bool TIGHT>
 __device__ void rle_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t nrows, uint32_t* wsm,
                         uint32_t* err) {
     const uint32_t lane = threadIdx.x & 31;
-    if (h.rows > (1u << 30)) {   // chunks hold at most 2^30 rows (the presum relies on it)
+    if (h.rows > (1u << 30)) {   // chunks hold at most 2^30 rows
         if (lane == 0) report(err, ZF_ECORRUPT, c.chunk_id);
         return;
     }
@@ -765,11 +764,11 @@ __device__ void rle_job(const ZfDevChunk& c, const Hdr& h, uint32_t r0, uint32_t
             T* dst = reinterpret_cast<T*>(c.dst) + rr;
             if (m <= kRleStageRuns) {
                 const uint8_t* b = bufs + (i % kRleStages) * bb;
-                rle_rows<T>(c, h, dst, reinterpret_cast<const uint32_t*>(b), rf & 3u,
+                rle_rows<T, TIGHT>(c, h, dst, reinterpret_cast<const uint32_t*>(b), rf & 3u,
                                 reinterpret_cast<const T*>(b + (kRleStageRuns + 4) * 4) + (rf & (VPER - 1)), bm, m,
                                 skip, nr, last, ns, lane, err);
             } else {
-                rle_rows<T>(c, h, dst, lens + (rf & ~3u), rf & 3u, vals + rf, bm, m, skip, nr, last, ns, lane,
+                rle_rows<T, TIGHT>(c, h, dst, lens + (rf & ~3u), rf & 3u, vals + rf, bm, m, skip, nr, last, ns, lane,
                                 err);
             }
         }

@@ -67,7 +67,7 @@ __device__ __forceinline__ void decode_mixed(const ZfDevChunk& c, const zfd::Hdr
                                              uint32_t* wsm, uint32_t* err) {
     switch (c.scheme * 4 + c.dtype) {
 #define ZF_CASE(S, D) \
-    case S * 4 + D: zfd::decode_one<S, D>(c, h, r0, nrows, wsm, err); break;
+    case S * 4 + D: zfd::decode_one<S, D, true>(c, h, r0, nrows, wsm, err); break;
         ZF_CASE(ZF_RAW, ZF_I32) ZF_CASE(ZF_RAW, ZF_I64) ZF_CASE(ZF_RAW, ZF_BYTES)
         ZF_CASE(ZF_FOR_BP, ZF_I32) ZF_CASE(ZF_FOR_BP, ZF_I64)
         ZF_CASE(ZF_DICT_BP, ZF_I32) ZF_CASE(ZF_DICT_BP, ZF_I64)
@@ -96,7 +96,7 @@ __device__ __forceinline__ void run_job(const LaunchArgs& a, uint32_t job, uint3
     }
     const uint32_t nrows = min(a.job_rows, c.rows - r0);
     if constexpr (SCHEME < 0) decode_mixed(c, h, r0, nrows, wsm, a.err);
-    else zfd::decode_one<SCHEME, DT>(c, h, r0, nrows, wsm, a.err);
+    else zfd::decode_one<SCHEME, DT, false>(c, h, r0, nrows, wsm, a.err);
 }
 
 // Specialized launches (one scheme and dtype): one warp job per warp, as

@@ -175,7 +175,7 @@ __device__ __forceinline__ void decode(const ZfDevChunk& c, const zfd::Hdr& h, u
                                        uint32_t* err) {
     switch (c.scheme * 4 + c.dtype) {
 #define ZF_CASE(S, D) \
-    case S * 4 + D: zfd::decode_one<S, D>(c, h, r0, nr, wsm, err); break;
+    case S * 4 + D: zfd::decode_one<S, D, true>(c, h, r0, nr, wsm, err); break;
         ZF_CASE(ZF_RAW, ZF_I32) ZF_CASE(ZF_RAW, ZF_I64) ZF_CASE(ZF_RAW, ZF_F64)
         ZF_CASE(ZF_FOR_BP, ZF_I32) ZF_CASE(ZF_FOR_BP, ZF_I64)
         ZF_CASE(ZF_DICT_BP, ZF_I32) ZF_CASE(ZF_DICT_BP, ZF_I64)
