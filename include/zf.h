@@ -9,7 +9,7 @@
  * patterns of Section 3.1:
  *   Fully-Parallel  -- FOR + bit-packing, dictionary + bit-packing, raw
  *   Group-Parallel  -- delta + bit-packing (block prefix scan), run-length
- *   Non-Parallel    -- LZ77 byte blocks, one warp per block
+ *   Non-Parallel    -- LZ77 byte blocks, one CTA or one warp per block
  *
  * Conventions for every call:
  *   - Every function returns zf_status; ZF_OK (0) is success.  No call
@@ -144,7 +144,10 @@ typedef struct {
     uint32_t tile_rows;       /* rows per warp job: a multiple of 1024, <= 16384 (0 = the
                                  class's tuned value, else 2048 for delta launches
                                  and 4096 for the others, halved down to 1024 while
-                                 a launch has fewer than 32 jobs per SM) */
+                                 a launch has fewer than 32 jobs per SM); LZ77, ANS and
+                                 string dictionaries that fit in shared memory (without
+                                 ZF_KCFG_BATCHED) have fixed jobs and read neither this
+                                 nor threads */
     uint32_t threads;         /* 128, 256 or 512 (0 = the class's tuned value, else 128) */
     uint32_t ctas_per_sm;     /* batched launch: persistent grid = ctas_per_sm x SM count (0 = occupancy limit) */
     uint32_t stage_bytes;     /* pipeline stage: compressed bytes per H2D copy + decode step (default 64 MiB) */

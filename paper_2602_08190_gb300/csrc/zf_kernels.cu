@@ -6,7 +6,10 @@
 //       any scheme and dtype, handed out by an atomic work queue; the last
 //       CTA to finish resets the queue so the launch can be replayed from a
 //       CUDA graph.
-// The LZ77 kernel (Non-Parallel pattern) is in zf_lz.cu.
+// LZ77 and ANS (Non-Parallel pattern) have their own kernels (zf_lz.cu,
+// zf_lz_cta.cu, zf_ans.cu), and so have string dictionaries that fit in shared
+// memory (zf_strdict_sm.cu); the string-dictionary code here decodes the others
+// and those of a batched launch.
 #include <cuda_runtime.h>
 
 #include <mutex>

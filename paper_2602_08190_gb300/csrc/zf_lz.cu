@@ -1,5 +1,6 @@
 // zf_lz.cu -- LZ77 decode, the Non-Parallel pattern of Section 3.1: blocks
-// of 64 KiB decode independently, each by one warp.  (Section 4 schedules one
+// of 64 KiB decode independently, here each by one warp (launches of few
+// blocks: by one CTA, zf_lz_cta.cu).  (Section 4 schedules one
 // thread per chunk; here the 32 lanes of a warp share one block, 32 tokens
 // at a time.)  Section 2.1 names LZ77; the block layout is this library's,
 // described with the format in zf.h.

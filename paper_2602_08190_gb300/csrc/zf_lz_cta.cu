@@ -71,14 +71,8 @@ struct LzSmem {
 __device__ __forceinline__ void warp_totals(const uint32_t* w, uint32_t lane, uint32_t warp, uint32_t& before,
                                             uint32_t& total) {
     const uint32_t x = lane < kLzWarps ? w[lane] : 0;
-    uint32_t s = x;
-#pragma unroll
-    for (uint32_t d = 1; d < kLzWarps; d <<= 1) {
-        const uint32_t a = __shfl_up_sync(kFull, s, d);
-        if (lane >= d) s += a;
-    }
-    before = __shfl_sync(kFull, s - x, warp);
-    total = __shfl_sync(kFull, s, kLzWarps - 1);
+    before = __reduce_add_sync(kFull, lane < warp ? x : 0u);
+    total = __reduce_add_sync(kFull, x);
 }
 
 __device__ __forceinline__ void prefetch_l2(const void* p) {

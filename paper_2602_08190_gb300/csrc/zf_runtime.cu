@@ -11,7 +11,7 @@
 // slot_copied) and decodes the stage into the caller's buffers.  Copies of
 // stage s+1.. run while stage s decodes, and the decodes of different stages
 // may run at once (stages are independent): a launch too small to fill the
-// GPU -- an LZ77 stage has one warp per 64 KiB block -- overlaps the next.
+// GPU -- an LZ77 stage has one CTA or warp per 64 KiB block -- overlaps the next.
 // The compute stream joins every decode stream at the end.  All descriptors
 // of a call are built on the host and copied once, ahead of the first stage.
 #include <cuda_runtime.h>
