@@ -325,13 +325,13 @@ def build_c3(zf, seed, text, scheme, chunk_mb):
     t, o = text
     if scheme == "lz77":
         return single(zf, "c3_lz77", f"non_parallel: {t.nbytes:,}-byte string column, Zipf(1.1) words from a 5,000-word "
-                      "vocabulary (3-12 letters), 1-8 words per row; LZ77 in 64 KiB blocks, one warp per block; "
+                      "vocabulary (3-12 letters), 1-8 words per row; LZ77 in 64 KiB blocks; "
                       "int32 offsets delta-packed", [((t, o), zf.ZF_LZ77, 0)],
                       "lz_kernel (+ the offsets' delta launch)")
     cb = int(chunk_mb * (1 << 20))
     return single(zf, "c3_strdict", f"group_parallel string dictionary: the same {t.nbytes:,}-byte text column as "
                   f"bit-packed codes into a sorted dictionary of tokens, {cb:,}-byte chunks; int32 offsets "
-                  "delta-packed", [((t, o), zf.ZF_STRDICT, cb)], "tiles_kernel<STRDICT, bytes> (+ the offsets' delta launch)")
+                  "delta-packed", [((t, o), zf.ZF_STRDICT, cb)], "strdict_kernel (+ the offsets' delta launch)")
 
 
 def build_ans(zf, seed, rows):

@@ -22,9 +22,9 @@ constexpr uint32_t kQueueWords = 2 + kAffinitySms + 6;
 
 // The chunk descriptors of a launch.  Up to kInlineChunks of them travel as
 // the kernel's parameters; more are read from a device array that the caller
-// has copied (a
-// copy ahead of the first kernel costs a call 3 to 4 us: 22.6 against 19.0 us
-// for 1M resident rows of FOR, 41.3 against 38.7 us for their transfer).
+// has copied (a copy ahead of the first kernel costs a call 3 to 4 us: 22.6
+// against 19.0 us for 1M resident rows of FOR, 41.3 against 38.7 us for their
+// transfer).
 constexpr uint32_t kInlineChunks = 64;
 struct ChunkArgs {
     const ZfDevChunk* dev;   // device array, or null: the descriptors are in `inl`

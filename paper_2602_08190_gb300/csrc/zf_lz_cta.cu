@@ -41,10 +41,10 @@ namespace {
 //   global memory.
 // What bounds it: the latency of a batch's chain of barriers, scans and
 // shared-memory lookups (14 batches of text per block).  Among thousands of
-// blocks it is bound by issue slots (64% busy), 228,000 warp instructions per
+// blocks it is bound by issue slots (64% busy), 229,000 warp instructions per
 // block of text: 40% of them to parse, place and store tokens, the rest in
 // about equal parts shortcuts with lookups of bytes.  Measured on GB300: 21
-// blocks of text (1.3 MB) 87 us per call with its host part, 548 us with one
+// blocks of text (1.3 MB) 85 us per call with its host part, 548 us with one
 // warp per block; 1,024 blocks 368 and 681 us.  Shortcuts whose steps were not
 // left for other tokens cost 27 us more of the 368.
 constexpr uint32_t kLzThreads = 512;
