@@ -109,6 +109,7 @@ __device__ __forceinline__ bool tile_tokens(const ZfDevChunk& c, const zfd::Hdr&
     const uint32_t* cw = reinterpret_cast<const uint32_t*>(c.blob + h.off[2]) + (uint64_t)tile * 32u * b;
     const uint32_t last_w = b ? (nt * b + 31) / 32 - 1 : 0;
     const uint8_t* winb = reinterpret_cast<const uint8_t*>(win);
+    __syncwarp();   // the warp's tile before may still be reading its last block there
     for (uint32_t w = lane; w < kWin; w += 32) win[w] = 0;
     uint32_t op = __ldg(tstart + tile);
     const uint32_t o1 = tile + 1 < ntiles ? __ldg(tstart + tile + 1) : h.rows;

@@ -56,3 +56,28 @@ def test_columns(name):
     finally:
         zf.zf_compressed_free(h)
         g.close()
+
+
+# Warps that decode several tiles one after another reuse their window: each
+# tile's last partial block has to be out before the next tile clears it.
+# 16M tokens are 15,625 tiles, four for each of the 32 warps of 152 CTAs.
+@pytest.mark.parametrize("lo,hi,tokens", [(1, 2, 20_000_000), (3, 4, 16_000_000)])
+def test_warps_of_several_tiles(lo, hi, tokens):
+    r = np.random.default_rng(lo)
+    words = np.full((7, hi), ord(" "), np.uint8)
+    lens = r.integers(lo, hi + 1, 7)
+    for i, n in enumerate(lens):
+        words[i, :n - 1] = 97 + i
+    pick = r.integers(0, 7, tokens)
+    t = words[pick].reshape(-1)[(np.arange(hi) < lens[pick][:, None]).reshape(-1)]
+    o = np.array([0, len(t)], np.int32)
+    col = zf.Column(t, o)
+    h = zf.zf_compress_host(zf.zf_plan(None, col, scheme=zf.ZF_STRDICT, chunk_rows=1 << 26), col)
+    g = Gpu()
+    try:
+        for _ in range(3):
+            got_t, got_o = g.decode([h], out_specs(t, o), resident=True)
+            assert np.array_equal(got_t, t) and np.array_equal(got_o, o)
+    finally:
+        zf.zf_compressed_free(h)
+        g.close()
