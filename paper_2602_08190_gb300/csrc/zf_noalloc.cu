@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) noalloc_decode(const 
                 }
                 if (ok) need = max(16u, (zfd::warp_smem((int)s_col.scheme, s_col.size, dc.bmax) + 15u) & ~15u);
                 else if (lane == 0) zfd::report(err, ZF_ECORRUPT, k);
+                __syncwarp();   // lanes may still be reading the job before's chunk there
                 if (lane == 0) {
                     s_dc[warp] = dc;
                     s_h[warp] = h;

@@ -105,3 +105,24 @@ def test_malformed_columns_are_refused_and_the_next_call_works():
         assert st == zf.ZF_OK and np.array_equal(out[:x.nbytes], x.view(np.uint8))
     assert _call(col, x.nbytes - 8)[0] == zf.ZF_EINVAL
     assert _call(col[:-16], x.nbytes)[0] == zf.ZF_ECORRUPT
+
+
+def test_warps_of_several_jobs_and_a_malformed_late_chunk():
+    """25M rows are 6,104 jobs of four tiles, more than one for the 4,864 warps
+    of a full grid on 152 SMs: a warp's second job takes its descriptor's place
+    while the first one's exceptions are patched, and in the malformed column
+    without any check that joins the warp before."""
+    n = 25_000_003
+    x = np.round(np.random.default_rng(6).integers(0, 1 << 20, n) / 100.0, 2)
+    x[::911] = np.nan                                              # exceptions all over the chunk
+    h = compress(x, zf.ZF_FLOAT2INT, 8192)
+    col = zf.zf_compressed_bytes(h)
+    zf.zf_compressed_free(h)
+    bad = bytearray(col)
+    last, = struct.unpack_from("<Q", col, 64 + 32 * (n // 8192))   # the last chunk's blob
+    struct.pack_into("<I", bad, last + 8, 1)                       # its rows
+    for _ in range(3):
+        st, out = _call(col, x.nbytes)
+        assert st == zf.ZF_OK and np.array_equal(out[:x.nbytes], x.view(np.uint8))
+        st, out = _call(bytes(bad), x.nbytes)
+        assert st == zf.ZF_ECORRUPT and (out[x.nbytes:] == SENTINEL).all()
