@@ -416,17 +416,16 @@ zf_status zf_mlp_get_scaling(const zf_mlp* net, float* mean, float* std);
  * device heap inside a call.  It calls no cudaMalloc, cudaFree or other
  * allocating routine and needs no zf_ctx.
  *
- * Its scratch (error word, finished-CTA count, result) is one fixed device
- * array of 32 bytes in the library, held by every GPU that loads the library
- * until the process exits.  Columns of more than 4096 chunks return ZF_EINVAL
+ * Its scratch (the calls' results) is one fixed device array of 512 bytes in
+ * the library, held by every GPU that loads the library until the process
+ * exits.  Columns of more than 4096 chunks return ZF_EINVAL
  * before anything is decoded.
  * The first call on a device looks up the array's device address, so make
  * that first call before any stream capture.  The call is synchronous: it
  * returns after the decode has finished and reports ZF_ECORRUPT if the
  * device checks of the stream failed (chunks that pass them may have been
- * decoded).  Every call on a device shares the
- * array; calls that overlap on the GPU, from several host threads or streams
- * at once, race -- serialize them.
+ * decoded).  Up to 64 calls may overlap on a device, from several host
+ * threads and on several streams.
  * Both pointers must be 16-byte aligned; `out_bytes` must hold all rows.
  * Returns ZF_EUNSUPPORTED for BYTES and ANS columns.  Besides the checks of the
  * other entry points' kernels, the device checks that each Float2Int chunk's

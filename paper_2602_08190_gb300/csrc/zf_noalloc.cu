@@ -7,13 +7,15 @@
 // front, a process whose memory budget is fixed by another runtime, or code
 // running inside a library call that may not grow the device heap.  Such a
 // caller passes its own input and output buffers; the only other memory the
-// decode needs (the error word, a count of finished CTAs and the result the
-// host reads) lives in the fixed-size device array below, which every GPU
-// that loads the library holds until the process exits.
+// decode needs (the result words the host reads) lives in the fixed-size
+// device array below, which every GPU that loads the library holds until the
+// process exits.
 //
-// The array is shared by all calls on a device; a launch leaves it ready for
-// the next.  Calls that overlap on the GPU -- from several host threads or
-// streams at once on the same device -- race on the array; serialize them.
+// Calls are numbered; call n uses result word n mod kSlots and writes it only
+// to report an error, as its number and the status.  Nothing is cleared
+// between calls: a word that names another call says nothing about this one,
+// whatever that call did, so calls may overlap (kSlots of them, before two
+// that fail could share a word).
 //
 // One launch does everything: every warp reads the column header, finds its
 // chunk by division (all chunks but the last have chunk_rows rows), checks
@@ -40,15 +42,16 @@ constexpr uint32_t kCtasPerSm = 8;
 constexpr uint32_t kSmem = 28 * 1024;         // a CTA's staging memory: four warps of up to 7 KB, fewer at a time of more
 constexpr uint32_t kJobTiles = 4;             // 1024-row tiles of a job at most
 constexpr int kMaxDevices = 64;
+constexpr uint32_t kSlots = 64;
 
-// [0] CTAs done, [1] error bits and [2] first failing chunk while a launch
-// runs; [3], [4] the same and [5] the column header's status when it is done.
-static __device__ uint32_t g_noalloc_ctrl[8] = {0, 0, 0xFFFFFFFFu, 0, 0, 0, 0, 0};
+// Result words: number << 8 | status of the last call that failed with it.
+static __device__ unsigned long long g_noalloc_slots[kSlots];
 
 std::mutex g_mu;
 struct Device {
-    void* ctrl = nullptr;   // device address of g_noalloc_ctrl (set once)
+    unsigned long long* slots = nullptr;   // device address of g_noalloc_slots (set once)
     int sms = 0;
+    uint64_t calls = 0;                    // so far
 } g_dev[kMaxDevices];
 
 struct Column {
@@ -189,20 +192,22 @@ __device__ __forceinline__ void decode(const ZfDevChunk& c, const zfd::Hdr& h, u
 // The jobs of a CTA share kSmem bytes: when the widest of them does not fit
 // four times, fewer warps decode at a time.
 __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) noalloc_decode(const uint8_t* col, uint64_t col_bytes,
-                                                                          uint8_t* out, uint64_t out_bytes) {
+                                                                          uint8_t* out, uint64_t out_bytes,
+                                                                          unsigned long long* slot, uint64_t call) {
     __shared__ uint4 smem4[kSmem / 16];
     __shared__ uint32_t s_need[kWarps];
     __shared__ Column s_col;
     __shared__ ZfDevChunk s_dc[kWarps];   // the warps' chunks, here and not in registers: 64 a thread are few
     __shared__ zfd::Hdr s_h[kWarps];      // for a kernel that decodes every scheme
     __shared__ uint32_t s_job_rows, s_per, s_njobs;   // rows of a job, jobs of a chunk, jobs of the column
-    uint32_t* ctrl = g_noalloc_ctrl;
-    uint32_t* err = ctrl + 1;
+    __shared__ uint32_t err[2];                       // error bits of the CTA's jobs and a chunk that failed
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         Column c;
         const zf_status st = read_column(col, col_bytes, out_bytes, c);
-        if (blockIdx.x == 0) ctrl[5] = (uint32_t)st;
+        if (blockIdx.x == 0 && st != ZF_OK) atomicMax(slot, (call << 8) | (uint32_t)st);
+        err[0] = 0;
+        err[1] = 0xFFFFFFFFu;
         s_njobs = 0;
         if (st == ZF_OK && c.n_rows) {
             const uint64_t tiles = (c.n_rows + 1023) / 1024, warps = (uint64_t)gridDim.x * kWarps;
@@ -253,17 +258,8 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) noalloc_decode(const 
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(&ctrl[0], 1u) == gridDim.x - 1) {
-            // the last CTA hands the result over and leaves the array ready for the next launch
-            __threadfence();
-            ctrl[3] = atomicExch(&ctrl[1], 0u);
-            ctrl[4] = atomicExch(&ctrl[2], 0xFFFFFFFFu);
-            ctrl[0] = 0;
-            __threadfence();
-        }
-    }
+    if (threadIdx.x == 0 && err[0])
+        atomicMax(slot, (call << 8) | (uint32_t)(err[0] & (1u << ZF_ECORRUPT) ? ZF_ECORRUPT : ZF_EINVAL));
 }
 
 }  // namespace
@@ -274,32 +270,31 @@ extern "C" zf_status zf_decompress_device_noalloc(const void* d_column, uint64_t
         return ZF_EINVAL;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return ZF_ECUDA;
-    Device d;
+    Device d;   // with this call's number
     {
         // first call on this device: look up the array's device address (the
         // host-side name of the array is not a device address)
         std::lock_guard<std::mutex> g(g_mu);
-        if (!g_dev[dev].ctrl) {
-            if (cudaGetSymbolAddress(&d.ctrl, g_noalloc_ctrl) != cudaSuccess || !d.ctrl ||
+        if (!g_dev[dev].slots) {
+            if (cudaGetSymbolAddress((void**)&d.slots, g_noalloc_slots) != cudaSuccess || !d.slots ||
                 cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || d.sms < 1) {
                 cudaGetLastError();
                 return ZF_ECUDA;
             }
             g_dev[dev] = d;
         }
+        g_dev[dev].calls++;
         d = g_dev[dev];
     }
     cudaStream_t s = (cudaStream_t)stream;
     // a column has at most out_bytes / 4 rows, or the kernel refuses it
     const uint64_t ctas = (out_bytes / 4096 + kWarps) / kWarps, most = (uint64_t)d.sms * kCtasPerSm;
     noalloc_decode<<<(unsigned)(ctas < most ? ctas : most), kWarps * 32, 0, s>>>(
-        (const uint8_t*)d_column, column_bytes, (uint8_t*)d_out, out_bytes);
+        (const uint8_t*)d_column, column_bytes, (uint8_t*)d_out, out_bytes, d.slots + d.calls % kSlots, d.calls);
     if (cudaGetLastError() != cudaSuccess) return ZF_ECUDA;
-    uint32_t r[3] = {0, 0, 0};   // error bits, first failing chunk, the header's status
-    if (cudaMemcpyAsync(r, (const uint8_t*)d.ctrl + 12, 12, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    unsigned long long r = 0;
+    if (cudaMemcpyAsync(&r, d.slots + d.calls % kSlots, sizeof(r), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return ZF_ECUDA;
-    if (r[2]) return (zf_status)r[2];
-    if (r[0] & (1u << ZF_ECORRUPT)) return ZF_ECORRUPT;
-    return r[0] ? ZF_EINVAL : ZF_OK;
+    return r >> 8 == d.calls ? (zf_status)(r & 0xFFu) : ZF_OK;
 }

@@ -126,3 +126,44 @@ def test_warps_of_several_jobs_and_a_malformed_late_chunk():
         assert st == zf.ZF_OK and np.array_equal(out[:x.nbytes], x.view(np.uint8))
         st, out = _call(bytes(bad), x.nbytes)
         assert st == zf.ZF_ECORRUPT and (out[x.nbytes:] == SENTINEL).all()
+
+
+def test_overlapping_calls_get_their_own_answers():
+    """Eight host threads call at once on streams of their own, half of them
+    with a malformed column; every call gets its own answer, and so does every
+    call after them."""
+    import threading
+
+    import torch
+    x = np.arange(200_000, dtype=np.int64) * 3
+    h = compress(x, zf.ZF_DELTA_BP, 8192)
+    good = zf.zf_compressed_bytes(h)
+    zf.zf_compressed_free(h)
+    bad = bytearray(good)
+    c5, = struct.unpack_from("<Q", good, 64 + 32 * 5)
+    struct.pack_into("<I", bad, c5 + 8, 1)
+    wrong = []
+
+    def worker(i):
+        stream = torch.cuda.Stream()
+        col = torch.frombuffer(bytearray(bad if i % 2 else good), dtype=torch.uint8).cuda()
+        out = torch.zeros(x.nbytes, dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        start.wait()
+        for _ in range(200):
+            st = zf.zf_decompress_device_noalloc(col.data_ptr(), col.numel(), out.data_ptr(), x.nbytes, stream.cuda_stream)
+            if st != (zf.ZF_ECORRUPT if i % 2 else zf.ZF_OK):
+                wrong.append((i, st))
+        if i % 2 == 0 and not np.array_equal(out.cpu().numpy(), x.view(np.uint8)):
+            wrong.append((i, "output"))
+
+    start = threading.Barrier(8)
+    threads = [threading.Thread(target=worker, args=(i,)) for i in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
+    for _ in range(70):                                            # more calls than result words
+        assert _call(bytes(bad), x.nbytes)[0] == zf.ZF_ECORRUPT
+        assert _call(good, x.nbytes)[0] == zf.ZF_OK
