@@ -423,9 +423,11 @@ zf_status zf_mlp_get_scaling(const zf_mlp* net, float* mean, float* std);
  * The first call on a device looks up the array's device address, so make
  * that first call before any stream capture.  The call is synchronous: it
  * returns after the decode has finished and reports ZF_ECORRUPT if the
- * device checks of the stream failed (chunks that pass them may have been
- * decoded).  Up to 64 calls may overlap on a device, from several host
- * threads and on several streams.
+ * device checks of the stream failed.  The header, the directory, every
+ * chunk's header and sections, the entries of delta blocks and the rows of
+ * Float2Int exceptions are checked before anything is decoded: where they are
+ * malformed, `d_out` is left as it was.  Up to 64 calls may
+ * overlap on a device, from several host threads and on several streams.
  * Both pointers must be 16-byte aligned; `out_bytes` must hold all rows.
  * Returns ZF_EUNSUPPORTED for BYTES and ANS columns.  Besides the checks of the
  * other entry points' kernels, the device checks that each Float2Int chunk's

@@ -17,19 +17,21 @@
 // whatever that call did, so calls may overlap (kSlots of them, before two
 // that fail could share a word).
 //
-// One launch does everything: every warp reads the column header, finds its
-// chunk by division (all chunks but the last have chunk_rows rows), checks
-// the chunk's directory entry and header and decodes its rows.  The host
-// waits once, for the result.  A header read by the host, a set-up kernel of
+// Two launches, one wait by the host: noalloc_check looks the whole column
+// over, noalloc_decode decodes it if nothing was found.  In both every warp
+// reads the column header and finds its chunk by division (all chunks but the
+// last have chunk_rows rows).  A header read by the host, a set-up kernel of
 // one CTA for the chunk descriptors (whose threads each walked a chunk's
 // delta entries) and a persistent decode launch took 46.3 us for 3M rows of
-// RLE and 220 us for 1M rows of delta in one chunk; this takes 26.8 and 27.7
-// us, most of it the host's wait.  From 8M rows on it is bound by DRAM: 33M
-// rows of Float2Int in 65,536-row chunks took 317 us and take 102 us (3.6
-// TB/s).
+// RLE and 220 us for 1M rows of delta in one chunk; this takes 28 us for
+// either, most of it the host's wait.  (One launch, in which a warp checked
+// only what it was about to decode, took 27 and 26.5 us, but had decoded
+// other chunks when one was found malformed.)  From 8M rows on it is bound by
+// DRAM: 33M rows of Float2Int in 65,536-row chunks took 317 us and take 102
+// us (3.6 TB/s).
 #include <cuda_runtime.h>
 
-#include <cstring>
+#include <algorithm>
 #include <mutex>
 
 #include "zf_decode.cuh"
@@ -43,6 +45,8 @@ constexpr uint32_t kSmem = 28 * 1024;         // a CTA's staging memory: four wa
 constexpr uint32_t kJobTiles = 4;             // 1024-row tiles of a job at most
 constexpr int kMaxDevices = 64;
 constexpr uint32_t kSlots = 64;
+constexpr uint32_t kRefused = 0x80;           // beside the status in a result word: nothing is decoded
+constexpr uint32_t kCheckTiles = 32;          // 1024-row tiles of a checking job: an entry of a delta block per lane
 
 // Result words: number << 8 | status of the last call that failed with it.
 static __device__ unsigned long long g_noalloc_slots[kSlots];
@@ -83,10 +87,23 @@ __device__ zf_status read_column(const uint8_t* col, uint64_t col_bytes, uint64_
     return c.n_rows * c.size > out_bytes ? ZF_EINVAL : ZF_OK;
 }
 
+// The warp jobs of a column, each of at most `rows` rows of one chunk.
+struct Jobs {
+    uint32_t rows, per, n;   // rows of a job, jobs of a chunk, jobs of the column
+};
+__device__ Jobs cut(const Column& c, uint32_t tiles) {
+    const uint32_t rows = 1024u * tiles, per = (c.chunk_rows + rows - 1) / rows;
+    const uint32_t last = (uint32_t)(c.n_rows - (uint64_t)(c.nch - 1) * c.chunk_rows);
+    return {rows, per, (c.nch - 1) * per + (last + rows - 1) / rows};   // a column of 2^32 jobs has 2^42 rows
+}
+
+__device__ __forceinline__ void post(unsigned long long* slot, uint64_t call, uint32_t status) {
+    atomicMax(slot, (call << 8) | status);
+}
+
 // Structural checks of chunk k (the host path makes the same checks before a
 // column is accepted) and its descriptor; false if it is malformed.  The
-// entries of delta blocks and Float2Int exceptions are checked by the jobs
-// that read them (job_ok).
+// entries of delta blocks and Float2Int exceptions are left to job_ok.
 __device__ bool chunk_ok(const uint8_t* col, const Column& c, uint32_t k, uint8_t* out, uint64_t out_bytes,
                          ZfDevChunk& dc, zfd::Hdr& h) {
     const uint8_t* d = col + 64 + 32ull * k;
@@ -143,35 +160,68 @@ __device__ bool chunk_ok(const uint8_t* col, const Column& c, uint32_t k, uint8_
     return false;
 }
 
-// The rest of a chunk's checks, shared by its jobs: delta block entries of
-// the job's rows (dc.bmax becomes the widest of them) and the job's share of
-// a Float2Int chunk's exception rows, which must be strictly increasing and
-// inside the chunk.
-__device__ bool job_ok(const zfd::Hdr& h, uint32_t r0, uint32_t nrows, uint32_t job_rows, ZfDevChunk& dc) {
+// Delta block entries of rows [r0, r0 + nrows) (32 blocks at most): true if
+// they lie inside the chunk; `widest` = the widest of them.
+__device__ bool delta_entries(const zfd::Hdr& h, uint32_t r0, uint32_t nrows, const ZfDevChunk& dc, uint32_t& widest) {
     const uint32_t lane = threadIdx.x & 31;
-    dc.bmax = (uint8_t)h.b;
+    uint32_t b = 0;
     bool ok = true;
-    if (dc.scheme == ZF_DELTA_BP) {
-        uint32_t b = 0;
-        if (lane * zf::kDeltaBlock < nrows) {
-            const uint8_t* e = dc.blob + h.off[0] + (uint64_t)(r0 / zf::kDeltaBlock + lane) * zf::kDeltaEntry;
-            const uint2 w = __ldg(reinterpret_cast<const uint2*>(e + 16));
-            const uint32_t mk = min(zf::kDeltaBlock, nrows - lane * zf::kDeltaBlock);
-            b = w.y & 0xFFu;
-            ok = b <= (dc.dtype == ZF_I32 ? 32u : 64u) && !(w.x & 15) &&
-                 (uint64_t)w.x + ((((uint64_t)mk * b + 7) / 8 + 15) & ~15ull) <= h.len[1];
-        }
-        dc.bmax = (uint8_t)__reduce_max_sync(0xFFFFFFFFu, b);
-    } else if (dc.scheme == ZF_FLOAT2INT) {
+    if (lane * zf::kDeltaBlock < nrows) {
+        const uint8_t* e = dc.blob + h.off[0] + (uint64_t)(r0 / zf::kDeltaBlock + lane) * zf::kDeltaEntry;
+        const uint2 w = __ldg(reinterpret_cast<const uint2*>(e + 16));
+        const uint32_t mk = min(zf::kDeltaBlock, nrows - lane * zf::kDeltaBlock);
+        b = w.y & 0xFFu;
+        ok = b <= (dc.dtype == ZF_I32 ? 32u : 64u) && !(w.x & 15) &&
+             (uint64_t)w.x + ((((uint64_t)mk * b + 7) / 8 + 15) & ~15ull) <= h.len[1];
+    }
+    widest = __reduce_max_sync(0xFFFFFFFFu, b);
+    return __all_sync(0xFFFFFFFFu, ok);
+}
+
+// The rest of a chunk's checks, shared by its jobs: delta block entries of
+// the job's rows and the job's share of a Float2Int chunk's exception rows,
+// which must be strictly increasing and inside the chunk.
+__device__ bool job_ok(const zfd::Hdr& h, uint32_t r0, uint32_t nrows, uint32_t job_rows, const ZfDevChunk& dc) {
+    uint32_t widest;
+    if (dc.scheme == ZF_DELTA_BP) return delta_entries(h, r0, nrows, dc, widest);
+    bool ok = true;
+    if (dc.scheme == ZF_FLOAT2INT) {
         const uint64_t jobs = (dc.rows + job_rows - 1) / job_rows, j = r0 / job_rows;
         const uint32_t z = (uint32_t)((j + 1) * h.n_aux / jobs);
         const uint32_t* er = reinterpret_cast<const uint32_t*>(dc.blob + h.off[1]);
-        for (uint32_t i = (uint32_t)(j * h.n_aux / jobs) + lane; i < z; i += 32) {
+        for (uint32_t i = (uint32_t)(j * h.n_aux / jobs) + (threadIdx.x & 31); i < z; i += 32) {
             const uint32_t x = __ldg(er + i);
             ok &= x < dc.rows && (i == 0 || x > __ldg(er + i - 1));
         }
     }
     return __all_sync(0xFFFFFFFFu, ok);
+}
+
+// Checks every chunk of the column; what it finds is in the call's result word
+// before noalloc_decode starts.  What bounds it: the latency of a chain of four
+// reads (column header, directory entry, chunk header, block entries).
+__global__ void __launch_bounds__(kWarps * 32) noalloc_check(const uint8_t* col, uint64_t col_bytes, uint8_t* out,
+                                                             uint64_t out_bytes, unsigned long long* slot,
+                                                             uint64_t call) {
+    __shared__ Column s_col;
+    __shared__ Jobs s_jobs;
+    if (threadIdx.x == 0) {
+        Column c;
+        const zf_status st = read_column(col, col_bytes, out_bytes, c);
+        if (blockIdx.x == 0 && st != ZF_OK) post(slot, call, kRefused | (uint32_t)st);
+        s_jobs = st == ZF_OK && c.n_rows ? cut(c, kCheckTiles) : Jobs{1, 1, 0};
+        s_col = c;
+    }
+    __syncthreads();
+    for (uint32_t job = blockIdx.x * kWarps + (threadIdx.x >> 5); job < s_jobs.n; job += gridDim.x * kWarps) {
+        ZfDevChunk dc{};
+        zfd::Hdr h{};
+        const uint32_t r0 = (job % s_jobs.per) * s_jobs.rows;
+        if (!chunk_ok(col, s_col, job / s_jobs.per, out, out_bytes, dc, h) ||
+            !job_ok(h, r0, min(s_jobs.rows, dc.rows - r0), s_jobs.rows, dc)) {
+            if ((threadIdx.x & 31) == 0) post(slot, call, kRefused | ZF_ECORRUPT);
+        }
+    }
 }
 
 __device__ __forceinline__ void decode(const ZfDevChunk& c, const zfd::Hdr& h, uint32_t r0, uint32_t nr, uint32_t* wsm,
@@ -199,67 +249,60 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) noalloc_decode(const 
     __shared__ Column s_col;
     __shared__ ZfDevChunk s_dc[kWarps];   // the warps' chunks, here and not in registers: 64 a thread are few
     __shared__ zfd::Hdr s_h[kWarps];      // for a kernel that decodes every scheme
-    __shared__ uint32_t s_job_rows, s_per, s_njobs;   // rows of a job, jobs of a chunk, jobs of the column
-    __shared__ uint32_t err[2];                       // error bits of the CTA's jobs and a chunk that failed
+    __shared__ Jobs s_jobs;
+    __shared__ uint32_t err[2];           // error bits of the CTA's jobs and a chunk that failed
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         Column c;
         const zf_status st = read_column(col, col_bytes, out_bytes, c);
-        if (blockIdx.x == 0 && st != ZF_OK) atomicMax(slot, (call << 8) | (uint32_t)st);
+        const unsigned long long found = __ldcg(slot);
         err[0] = 0;
         err[1] = 0xFFFFFFFFu;
-        s_njobs = 0;
-        if (st == ZF_OK && c.n_rows) {
+        s_jobs = Jobs{1, 1, 0};
+        if (st == ZF_OK && c.n_rows && !(found >> 8 == call && (found & kRefused))) {
             const uint64_t tiles = (c.n_rows + 1023) / 1024, warps = (uint64_t)gridDim.x * kWarps;
-            const uint32_t most = (uint32_t)min((unsigned long long)kJobTiles, (unsigned long long)((tiles + warps - 1) / warps));
-            const uint32_t rows = 1024u * most, per = (c.chunk_rows + rows - 1) / rows;
-            const uint32_t last = (uint32_t)(c.n_rows - (uint64_t)(c.nch - 1) * c.chunk_rows);
-            s_job_rows = rows;
-            s_per = per;
-            s_njobs = (c.nch - 1) * per + (last + rows - 1) / rows;   // a column of 2^32 jobs has 2^42 rows
+            s_jobs = cut(c, (uint32_t)min((unsigned long long)kJobTiles, (unsigned long long)((tiles + warps - 1) / warps)));
         }
         s_col = c;
     }
     __syncthreads();
-    {
-        for (uint32_t base = blockIdx.x * kWarps; base < s_njobs; base += gridDim.x * kWarps) {
-            const uint32_t job = base + warp;
-            uint32_t need = 0, r0 = 0, nr = 0;
-            ZfDevChunk dc{};
-            zfd::Hdr h{};
-            if (job < s_njobs) {
-                const uint32_t k = job / s_per;
-                r0 = (job % s_per) * s_job_rows;
-                bool ok = chunk_ok(col, s_col, k, out, out_bytes, dc, h);
-                if (ok) {
-                    nr = min(s_job_rows, dc.rows - r0);
-                    ok = job_ok(h, r0, nr, s_job_rows, dc);
-                }
-                if (ok) need = max(16u, (zfd::warp_smem((int)s_col.scheme, s_col.size, dc.bmax) + 15u) & ~15u);
-                else if (lane == 0) zfd::report(err, ZF_ECORRUPT, k);
-                __syncwarp();   // lanes may still be reading the job before's chunk there
-                if (lane == 0) {
-                    s_dc[warp] = dc;
-                    s_h[warp] = h;
-                }
+    for (uint32_t base = blockIdx.x * kWarps; base < s_jobs.n; base += gridDim.x * kWarps) {
+        const uint32_t job = base + warp;
+        uint32_t need = 0, r0 = 0, nr = 0;
+        ZfDevChunk dc{};
+        zfd::Hdr h{};
+        if (job < s_jobs.n) {
+            const uint32_t k = job / s_jobs.per;
+            r0 = (job % s_jobs.per) * s_jobs.rows;
+            if (chunk_ok(col, s_col, k, out, out_bytes, dc, h)) {   // as noalloc_check found it
+                nr = min(s_jobs.rows, dc.rows - r0);
+                uint32_t widest = h.b;
+                if (s_col.scheme == ZF_DELTA_BP) delta_entries(h, r0, nr, dc, widest);
+                dc.bmax = (uint8_t)widest;
+                need = max(16u, (zfd::warp_smem((int)s_col.scheme, s_col.size, dc.bmax) + 15u) & ~15u);
             }
-            __syncthreads();
-            if (lane == 0) s_need[warp] = need;
-            __syncthreads();
-            uint32_t most = 16;
+            __syncwarp();   // lanes may still be reading the job before's chunk there
+            if (lane == 0) {
+                s_dc[warp] = dc;
+                s_h[warp] = h;
+            }
+        }
+        __syncthreads();
+        if (lane == 0) s_need[warp] = need;
+        __syncthreads();
+        uint32_t most = 16;
 #pragma unroll
-            for (uint32_t w = 0; w < kWarps; w++) most = max(most, s_need[w]);
-            const uint32_t at_once = min(kWarps, kSmem / most);
-            for (uint32_t g = 0; g < kWarps; g += at_once) {
-                if (need && warp >= g && warp < g + at_once)
-                    decode(s_dc[warp], s_h[warp], r0, nr, reinterpret_cast<uint32_t*>(smem4) + (warp - g) * (most / 4), err);
-                if (at_once < kWarps) __syncthreads();
-            }
+        for (uint32_t w = 0; w < kWarps; w++) most = max(most, s_need[w]);
+        const uint32_t at_once = min(kWarps, kSmem / most);
+        for (uint32_t g = 0; g < kWarps; g += at_once) {
+            if (need && warp >= g && warp < g + at_once)
+                decode(s_dc[warp], s_h[warp], r0, nr, reinterpret_cast<uint32_t*>(smem4) + (warp - g) * (most / 4), err);
+            if (at_once < kWarps) __syncthreads();
         }
     }
     __syncthreads();
     if (threadIdx.x == 0 && err[0])
-        atomicMax(slot, (call << 8) | (uint32_t)(err[0] & (1u << ZF_ECORRUPT) ? ZF_ECORRUPT : ZF_EINVAL));
+        post(slot, call, err[0] & (1u << ZF_ECORRUPT) ? ZF_ECORRUPT : ZF_EINVAL);
 }
 
 }  // namespace
@@ -287,14 +330,18 @@ extern "C" zf_status zf_decompress_device_noalloc(const void* d_column, uint64_t
         d = g_dev[dev];
     }
     cudaStream_t s = (cudaStream_t)stream;
-    // a column has at most out_bytes / 4 rows, or the kernel refuses it
-    const uint64_t ctas = (out_bytes / 4096 + kWarps) / kWarps, most = (uint64_t)d.sms * kCtasPerSm;
-    noalloc_decode<<<(unsigned)(ctas < most ? ctas : most), kWarps * 32, 0, s>>>(
-        (const uint8_t*)d_column, column_bytes, (uint8_t*)d_out, out_bytes, d.slots + d.calls % kSlots, d.calls);
+    // a column has at most out_bytes / 4 rows, or the kernels refuse it
+    const uint64_t ctas = (out_bytes / 4096 + kWarps) / kWarps, sms = (uint64_t)d.sms;
+    const uint8_t* col = (const uint8_t*)d_column;
+    uint8_t* out = (uint8_t*)d_out;
+    unsigned long long* slot = d.slots + d.calls % kSlots;
+    noalloc_check<<<(unsigned)std::min(ctas, 2 * sms), kWarps * 32, 0, s>>>(col, column_bytes, out, out_bytes, slot, d.calls);
+    noalloc_decode<<<(unsigned)std::min(ctas, kCtasPerSm * sms), kWarps * 32, 0, s>>>(col, column_bytes, out, out_bytes, slot,
+                                                                                      d.calls);
     if (cudaGetLastError() != cudaSuccess) return ZF_ECUDA;
     unsigned long long r = 0;
-    if (cudaMemcpyAsync(&r, d.slots + d.calls % kSlots, sizeof(r), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    if (cudaMemcpyAsync(&r, slot, sizeof(r), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return ZF_ECUDA;
-    return r >> 8 == d.calls ? (zf_status)(r & 0xFFu) : ZF_OK;
+    return r >> 8 == d.calls ? (zf_status)(r & 0xFFu & ~kRefused) : ZF_OK;
 }

@@ -167,3 +167,34 @@ def test_overlapping_calls_get_their_own_answers():
     for _ in range(70):                                            # more calls than result words
         assert _call(bytes(bad), x.nbytes)[0] == zf.ZF_ECORRUPT
         assert _call(good, x.nbytes)[0] == zf.ZF_OK
+
+
+@pytest.mark.parametrize("scheme", ["for", "dict", "delta", "rle", "float2int", "raw"])
+@pytest.mark.parametrize("where", ["header", "sections"])
+def test_nothing_is_decoded_of_a_malformed_column(scheme, where):
+    """A fault in the last of many chunks leaves the whole output as it was."""
+    n = 70 * 8192 + 5
+    make = {"for": (lambda: _wide(n, 17, np.int32), zf.ZF_FOR_BP), "dict": (lambda: _wide(n, 6, np.int64), zf.ZF_DICT_BP),
+            "delta": (lambda: W.sorted_keys(4, n), zf.ZF_DELTA_BP), "rle": (lambda: W.dates_rle(4, n), zf.ZF_RLE),
+            "float2int": (lambda: np.where(np.arange(n) % 5 == 0, np.nan, W.decimal_prices(1, 7, 0, n)), zf.ZF_FLOAT2INT),
+            "raw": (lambda: _wide(n, 64, np.int64), zf.ZF_RAW)}[scheme]
+    x = make[0]()
+    h = compress(x, make[1], 8192)
+    col = zf.zf_compressed_bytes(h)
+    zf.zf_compressed_free(h)
+    bad = bytearray(col)
+    blob, = struct.unpack_from("<Q", col, 64 + 32 * 70)            # the last chunk, 5 rows
+    off = struct.unpack_from("<III", col, blob + 24)
+    if where == "header":
+        struct.pack_into("<I", bad, blob, 0)
+    elif scheme == "delta":
+        struct.pack_into("<B", bad, blob + off[0] + 20, 65)        # a block wider than the type
+    elif scheme == "float2int":
+        struct.pack_into("<I", bad, blob + off[1], 5)              # an exception past the chunk
+    else:
+        length, = struct.unpack_from("<I", col, blob + 36)
+        struct.pack_into("<I", bad, blob + 36, length + 4)         # the first section's length
+    st, out = _call(bytes(bad), x.nbytes)
+    assert st == zf.ZF_ECORRUPT and (out == SENTINEL).all()
+    st, out = _call(col, x.nbytes)
+    assert st == zf.ZF_OK and np.array_equal(out[:x.nbytes], x.view(np.uint8))
