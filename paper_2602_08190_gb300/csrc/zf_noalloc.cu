@@ -26,9 +26,9 @@
 // RLE and 220 us for 1M rows of delta in one chunk; this takes 28 us for
 // either, most of it the host's wait.  (One launch, in which a warp checked
 // only what it was about to decode, took 27 and 26.5 us, but had decoded
-// other chunks when one was found malformed.)  From 8M rows on it is bound by
-// DRAM: 33M rows of Float2Int in 65,536-row chunks took 317 us and take 102
-// us (3.6 TB/s).
+// other chunks when one was found malformed.)  33M rows of Float2Int in
+// 65,536-row chunks took 317 us and take 102 us: about 25 us of launches and
+// wait, as for the smallest column, then 4.7 TB/s.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,6 +40,10 @@ namespace {
 
 constexpr uint32_t kNoallocMaxChunks = 4096;
 constexpr uint32_t kWarps = 4;                // warps per CTA
+// Seven CTAs fit an SM beside one another (29 KB of shared memory each); the
+// eighth of a full grid starts as one of them ends.  A grid of seven (33M wide
+// differences 3% faster, 33M narrow FOR 4% slower) and eight of 27,632 bytes
+// that do fit (the wide differences 5% slower) measured the same elsewhere.
 constexpr uint32_t kCtasPerSm = 8;
 constexpr uint32_t kSmem = 28 * 1024;         // a CTA's staging memory: four warps of up to 7 KB, fewer at a time of more
 constexpr uint32_t kJobTiles = 4;             // 1024-row tiles of a job at most
