@@ -610,6 +610,7 @@ struct zf_mlp {
     uint8_t* data = nullptr;  // zf_mlp_train's and zf_mlp_predict's rows on the device, kept for the next call
     size_t data_cap = 0;
     std::mutex data_mu;       // held by the calls that use `data`
+    cudaEvent_t copied[2] = {nullptr, nullptr};   // zf_mlp_train's uploads, two in turn: the copy has read its source
     int cluster = -1;         // whether mlp_train_cluster fits the device (-1: not asked yet)
     uint32_t step = 0;
     // input standardization (x - mean) / std, fitted by zf_mlp_train on its
@@ -714,7 +715,9 @@ zf_status zf_mlp_create(int device, uint64_t seed, zf_mlp** out) {
     auto* n = new zf_mlp();
     n->device = device;
     if (cudaMalloc(&n->p, NP * sizeof(float)) != cudaSuccess || cudaMalloc(&n->m, NP * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&n->v, NP * sizeof(float)) != cudaSuccess) {
+        cudaMalloc(&n->v, NP * sizeof(float)) != cudaSuccess ||
+        cudaEventCreateWithFlags(&n->copied[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&n->copied[1], cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         zf_mlp_destroy(n);
         return ZF_ENOMEM;
@@ -746,6 +749,8 @@ zf_status zf_mlp_destroy(zf_mlp* n) {
     cudaSetDevice(n->device);
     for (void* q : {(void*)n->p, (void*)n->m, (void*)n->v, (void*)n->part, (void*)n->data})
         if (q) cudaFree(q);
+    for (cudaEvent_t e : n->copied)
+        if (e) cudaEventDestroy(e);
     delete n;
     return ZF_OK;
 }
@@ -829,6 +834,7 @@ zf_status zf_mlp_train(zf_mlp* n, const float* h_x, const int32_t* h_y, const ui
                          {(void**)&dx, (void**)&dy, (void**)&dm, (void**)&dord, (void**)&dl});
     if (st) return st;
     auto done = [&](zf_status s) {
+        if (s != ZF_OK) cudaDeviceSynchronize();   // uploads in flight read this call's memory
         release_large(n);
         return s;
     };
@@ -862,22 +868,30 @@ zf_status zf_mlp_train(zf_mlp* n, const float* h_x, const int32_t* h_y, const ui
     }
     std::vector<uint64_t> hash(count + 1);   // of the counter generator, the same every epoch
     for (uint32_t i = 2; i <= count; i++) hash[i] = splitmix(i);
-    std::vector<uint32_t> up(words);
+    // An upload may still be reading its host buffer when cudaMemcpyAsync returns: two take turns, and one is refilled
+    // after the event behind its copy
+    std::vector<uint32_t> up[2];
+    uint32_t uploads = 0;
     std::vector<float> losses((size_t)back * steps);
     uint32_t group = 1;                      // the first launch starts after one shuffle, later ones are larger
     for (uint32_t e0 = 0; e0 < epochs; e0 += back) {
         const uint32_t e1 = std::min(epochs, e0 + back);
         for (uint32_t e = e0; e < e1;) {
             const uint32_t ne = std::min(std::min(group, most), e1 - e);
+            std::vector<uint32_t>& buf = up[uploads & 1];
+            const cudaEvent_t copied = n->copied[uploads & 1];
+            if (uploads >= 2 && cudaEventSynchronize(copied) != cudaSuccess) return done(ZF_ECUDA);
+            uploads++;
+            buf.resize(words);
             for (uint32_t q = 0; q < ne; q++) {
-                uint32_t* order = up.data() + (size_t)q * count;
+                uint32_t* order = buf.data() + (size_t)q * count;
                 std::iota(order, order + count, 0u);
                 for (uint32_t i = count; i > 1; i--) {   // Fisher-Yates with the counter generator
                     const uint32_t j = (uint32_t)(unit_of(splitmix((seed + e + q) ^ hash[i])) * i);
                     std::swap(order[i - 1], order[std::min(j, i - 1)]);
                 }
             }
-            float* c = reinterpret_cast<float*>(up.data() + (size_t)ne * count);
+            float* c = reinterpret_cast<float*>(buf.data() + (size_t)ne * count);
             const uint32_t ns = ne * steps;
             for (uint32_t k = 0; k < ns; k++) {
                 n->step++;
@@ -885,8 +899,9 @@ zf_status zf_mlp_train(zf_mlp* n, const float* h_x, const int32_t* h_y, const ui
                 c[ns + k] = (float)(1.0 - std::pow(0.999, (double)n->step));
             }
             float* dloss = dl + (size_t)(e - e0) * steps;
-            if (cudaMemcpyAsync(dord, up.data(), ((size_t)ne * count + 2 * (size_t)ns) * sizeof(uint32_t), cudaMemcpyHostToDevice, 0) !=
-                cudaSuccess)
+            if (cudaMemcpyAsync(dord, buf.data(), ((size_t)ne * count + 2 * (size_t)ns) * sizeof(uint32_t), cudaMemcpyHostToDevice,
+                                0) != cudaSuccess ||
+                cudaEventRecord(copied, 0) != cudaSuccess)
                 return done(ZF_ECUDA);
             if (cluster) {
                 args.order = dord;

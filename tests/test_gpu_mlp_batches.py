@@ -91,3 +91,23 @@ def test_training_matches_float64(count, batch, epochs):
         assert d.max() <= 6e-3 and d.mean() <= 4e-5
     finally:
         zf.zf_mlp_destroy(net)
+
+
+# The epochs of a call are shuffled and uploaded in groups of 1, 2, 4, ... and
+# each group runs in one launch (batches above 512: an epoch per upload); one
+# epoch at a time nothing is uploaded twice and no launch holds two epochs.
+# The arithmetic is the same, so the bits are.
+@pytest.mark.parametrize("count,batch,epochs", [(300, 256, 8), (64, 64, 70), (700, 300, 9), (1100, 512, 8), (516, 257, 5), (1100, 600, 7),
+                                                (20_000, 500, 12), (20_000, 700, 6)])
+def test_a_call_trains_as_its_epochs_one_by_one(count, batch, epochs):
+    X, y, mask = _batch(count + 1, count)
+    mask = mask.astype(np.uint8)
+    a, b = zf.zf_mlp_create(0, 4), zf.zf_mlp_create(0, 4)
+    try:
+        together = zf.zf_mlp_train(a, X, y, mask, epochs, batch, 1e-3, seed=17)
+        single = [zf.zf_mlp_train(b, X, y, mask, 1, batch, 1e-3, seed=17 + e)[0] for e in range(epochs)]
+        assert np.array_equal(together, np.array(single, together.dtype))
+        assert np.array_equal(zf.zf_mlp_get_params(a), zf.zf_mlp_get_params(b))
+    finally:
+        zf.zf_mlp_destroy(a)
+        zf.zf_mlp_destroy(b)
