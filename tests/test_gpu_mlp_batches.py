@@ -1,6 +1,6 @@
 """The selector network's batch kernels at the sizes where their tiles of
 eight samples begin and end, and training inside one cluster (batches of up to
-512 samples, eight ranks of 32 at a time) or as launches per step, against the
+512 samples, sixteen ranks of 16 at a time) or as launches per step, against the
 float64 oracle with the same sample order."""
 import numpy as np
 import pytest
@@ -66,7 +66,7 @@ def _order(n, seed):
     return o
 
 
-@pytest.mark.parametrize("count,batch,epochs", [(5, 8, 3), (100, 33, 2), (300, 256, 2), (257, 257, 2), (512, 512, 2), (1100, 513, 2), (600, 4000, 3)])
+@pytest.mark.parametrize("count,batch,epochs", [(5, 8, 3), (100, 33, 2), (300, 256, 2), (257, 257, 2), (512, 512, 2), (1100, 512, 2), (516, 257, 2), (700, 300, 2), (1100, 513, 2), (600, 4000, 3)])
 def test_training_matches_float64(count, batch, epochs):
     X, y, mask = _batch(count, count)
     net = zf.zf_mlp_create(0, 21)
