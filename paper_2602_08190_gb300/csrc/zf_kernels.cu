@@ -17,6 +17,7 @@
 
 #include "zf_decode.cuh"
 #include "zf_launch.h"
+#include "zf_once.h"
 
 namespace {
 
@@ -195,8 +196,11 @@ KernelFn<INL> pick(int scheme, int dtype) {
 
 struct OccKey {
     void* fn;
+    int device;
     uint32_t smem, threads;
-    bool operator==(const OccKey& o) const { return fn == o.fn && smem == o.smem && threads == o.threads; }
+    bool operator==(const OccKey& o) const {
+        return fn == o.fn && device == o.device && smem == o.smem && threads == o.threads;
+    }
 };
 struct OccHash {
     size_t operator()(const OccKey& k) const {
@@ -205,7 +209,7 @@ struct OccHash {
 };
 std::mutex g_occ_mu;
 std::unordered_map<OccKey, int, OccHash> g_occ;
-std::unordered_map<void*, bool> g_attr_set;
+zf::OncePerDevice g_smem_allowed;
 
 template <bool INL, class Chunks>
 cudaError_t launch(const zf::TileLaunch& L, const Chunks& chunks, cudaStream_t s) {
@@ -217,24 +221,23 @@ cudaError_t launch(const zf::TileLaunch& L, const Chunks& chunks, cudaStream_t s
     default: return cudaErrorInvalidValue;
     }
     if (!fn) return cudaErrorInvalidValue;
-    int per_sm = (int)L.ctas_per_sm;
+    int per_sm = (int)L.ctas_per_sm, dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    // allow the largest dynamic shared memory any launch of this kernel may ask for
+    e = g_smem_allowed(dev, (const void*)fn, [&] {
+        int optin = 0;
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)(2 * 1024));
+    });
+    if (e != cudaSuccess) return e;
     {
         std::lock_guard<std::mutex> g(g_occ_mu);
-        if (!g_attr_set.count((void*)fn)) {
-            // allow the largest dynamic shared memory any launch of this kernel may ask for
-            int dev = 0, optin = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 optin - (int)(2 * 1024));
-            if (e != cudaSuccess) return e;
-            g_attr_set[(void*)fn] = true;
-        }
-        OccKey key{(void*)fn, L.smem, L.threads};
+        OccKey key{(void*)fn, dev, L.smem, L.threads};
         auto it = g_occ.find(key);
         if (it == g_occ.end()) {
             int occ = 0;
-            cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, (int)L.threads, L.smem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, (int)L.threads, L.smem);
             if (e != cudaSuccess) return e;
             it = g_occ.emplace(key, occ).first;
         }

@@ -3,10 +3,9 @@
 // one warp takes for it (zf_lz.cu, which says where the line lies).
 #include <cuda_runtime.h>
 
-#include <mutex>
-
 #include "zf_device.cuh"
 #include "zf_launch.h"
+#include "zf_once.h"
 
 namespace {
 
@@ -379,9 +378,7 @@ __global__ void __launch_bounds__(kLzThreads, 2) lz_cta_kernel(const __grid_cons
     lz_block(c, *reinterpret_cast<LzSmem*>(smem4), err);
 }
 
-constexpr int kMaxDevices = 64;
-std::mutex g_mu;
-bool g_attr_set[kMaxDevices];   // shared-memory attribute of lz_cta_kernel set on the device
+zf::OncePerDevice g_smem_allowed;
 
 }  // namespace
 
@@ -391,14 +388,10 @@ cudaError_t launch_lz_cta(const ChunkArgs& chunks, uint32_t* err, cudaStream_t s
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    {
-        std::lock_guard<std::mutex> g(g_mu);
-        if (dev >= kMaxDevices || !g_attr_set[dev]) {
-            e = cudaFuncSetAttribute(lz_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LzSmem));
-            if (e != cudaSuccess) return e;
-            if (dev < kMaxDevices) g_attr_set[dev] = true;
-        }
-    }
+    e = g_smem_allowed(dev, (const void*)lz_cta_kernel, [] {
+        return cudaFuncSetAttribute(lz_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LzSmem));
+    });
+    if (e != cudaSuccess) return e;
     lz_cta_kernel<<<chunks.n, kLzThreads, sizeof(LzSmem), s>>>(chunks, err);
     return cudaGetLastError();
 }

@@ -17,10 +17,9 @@
 // now: 256 MB 374 and 222 us (1.5 TB/s), 64 MB 146 and 104, 8 MB 86 and 54.
 #include <cuda_runtime.h>
 
-#include <mutex>
-
 #include "zf_decode.cuh"
 #include "zf_launch.h"
+#include "zf_once.h"
 
 namespace {
 
@@ -222,9 +221,7 @@ __global__ void __launch_bounds__(kThreads, 1) strdict_kernel(const __grid_const
     }
 }
 
-constexpr int kMaxDevices = 64;
-std::mutex g_mu;
-bool g_attr_set[kMaxDevices];
+zf::OncePerDevice g_smem_allowed;
 
 }  // namespace
 
@@ -238,15 +235,11 @@ cudaError_t launch_strdict(const ZfDevChunk* chunks, const ZfDevChunk* host, uin
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    {
-        std::lock_guard<std::mutex> g(g_mu);
-        if (dev >= kMaxDevices || !g_attr_set[dev]) {
-            e = cudaFuncSetAttribute(strdict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(kWarps * kWin * 4u + strdict_smem_limit()));
-            if (e != cudaSuccess) return e;
-            if (dev < kMaxDevices) g_attr_set[dev] = true;
-        }
-    }
+    e = g_smem_allowed(dev, (const void*)strdict_kernel, [] {
+        return cudaFuncSetAttribute(strdict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kWarps * kWin * 4u + strdict_smem_limit()));
+    });
+    if (e != cudaSuccess) return e;
     const uint32_t grid = ntiles < (uint32_t)num_sms ? ntiles : (uint32_t)num_sms;
     strdict_kernel<<<grid, kThreads, kWarps * kWin * 4u + ((dict_bytes + 15u) & ~15u), s>>>(
         Args{ChunkArgs(chunks, host, nchunks), ntiles, (dict_bytes + 15u) & ~15u, err});
