@@ -146,7 +146,8 @@ typedef struct {
                                  and 4096 for the others, halved down to 1024 while
                                  a launch has fewer than 32 jobs per SM); LZ77, ANS and
                                  string dictionaries that fit in shared memory (without
-                                 ZF_KCFG_BATCHED) have fixed jobs and read neither this
+                                 ZF_KCFG_BATCHED; not launches of many chunks of under
+                                 16,384 tokens) have fixed jobs and read neither this
                                  nor threads */
     uint32_t threads;         /* 128, 256 or 512 (0 = the class's tuned value, else 128) */
     uint32_t ctas_per_sm;     /* batched launch: persistent grid = ctas_per_sm x SM count (0 = occupancy limit) */

@@ -8,8 +8,8 @@
 //       CUDA graph.
 // LZ77 and ANS (Non-Parallel pattern) have their own kernels (zf_lz.cu,
 // zf_lz_cta.cu, zf_ans.cu), and so have string dictionaries that fit in shared
-// memory (zf_strdict_sm.cu); the string-dictionary code here decodes the others
-// and those of a batched launch.
+// memory (zf_strdict_sm.cu); the string-dictionary code here decodes the others,
+// those of a batched launch and launches of many short chunks.
 #include <cuda_runtime.h>
 
 #include <mutex>

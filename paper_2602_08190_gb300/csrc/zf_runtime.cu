@@ -255,13 +255,34 @@ struct Group {
 // say; zf_strdict_sm.cu); a larger one is read through L1 (zf_strdict.cuh).
 constexpr int kStrdictSmem = ZF_NSCHEMES;
 
+bool fits_shared(const zf::ChunkInfo& ch) { return ch.scheme == ZF_STRDICT && ch.dict_bytes <= zf::strdict_smem_limit(); }
+
+// Whether the dictionaries of works[b, e) that fit go to shared memory.  A CTA
+// lays a chunk's dictionary out with its 32 warps waiting (about 15 us), then
+// each takes a tile: where an SM gets many chunks of few tiles that wait is
+// what a launch takes.  Text of 5,000 words in chunks of 64 KiB (11 tiles),
+// through L1 and with shared memory: 1.3 MB 57 and 47 us, 16 MB 111 and 75,
+// 64 MB (6.7 chunks per SM) 169 and 181, 256 MB 519 and 602; in chunks of 128
+// KiB (22 tiles) 56 and 36, 108 and 59, 156 and 130, 455 and 365.
+constexpr uint32_t kShortChunkTiles = 16, kShortChunksPerSm = 4;
+bool strdict_shared(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_t e) {
+    uint64_t n = 0, tiles = 0;
+    for (size_t i = b; i < e; i++)
+        if (fits_shared(*w[i].ch)) {
+            n++;
+            tiles += (w[i].ch->units + zf::kStrTile - 1) / zf::kStrTile;
+        }
+    return tiles >= n * kShortChunkTiles || n <= (uint64_t)ctx->num_sms * kShortChunksPerSm;
+}
+
 // The launch a chunk belongs to: LZ77, ANS and string dictionaries in shared
-// memory have kernels of their own, batched or not.
-std::pair<int, int> group_key(const zf::ChunkInfo& ch, bool batched) {
+// memory (`shared`: where they fit) have kernels of their own, the first two
+// batched or not.
+std::pair<int, int> group_key(const zf::ChunkInfo& ch, bool batched, bool shared) {
     if (ch.scheme == ZF_LZ77) return {ZF_LZ77, ZF_BYTES};
     if (ch.scheme == ZF_ANS) return {ch.scheme, ch.dtype};
     if (batched) return {-1, -1};
-    if (ch.scheme == ZF_STRDICT && ch.dict_bytes <= zf::strdict_smem_limit()) return {kStrdictSmem, ZF_BYTES};
+    if (shared && fits_shared(ch)) return {kStrdictSmem, ZF_BYTES};
     return {ch.scheme, ch.dtype};
 }
 
@@ -270,7 +291,7 @@ std::pair<int, int> group_key(const zf::ChunkInfo& ch, bool batched) {
 // three times per chunk and the vectors grew as they filled; it takes 185.
 void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_t e, const zf_kcfg& k,
                   std::vector<ZfDevChunk>& desc, std::vector<Group>& groups) {
-    const bool batched = k.flags & ZF_KCFG_BATCHED;
+    const bool batched = k.flags & ZF_KCFG_BATCHED, shared = strdict_shared(ctx, w, b, e);
     struct Key {
         std::pair<int, int> key;
         uint32_t bmax = 0;         // widest bit width of the group: its geometry class
@@ -281,7 +302,7 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
     std::vector<uint8_t> key_of(e - b);   // a call has few groups: at most one per scheme and type
     for (size_t i = b; i < e; i++) {
         const zf::ChunkInfo& ch = *w[i].ch;
-        const auto key = group_key(ch, batched);
+        const auto key = group_key(ch, batched, shared);
         size_t q = 0;
         while (q < keys.size() && keys[q].key != key) q++;
         if (q == keys.size()) keys.push_back({key});

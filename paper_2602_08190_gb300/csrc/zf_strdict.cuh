@@ -2,7 +2,8 @@
 // a byte column stored as bit-packed codes into a dictionary of tokens
 // (Section 2.1 dictionary encoding over the words of a text column, as
 // Section 5.3.1 does for the comment column), the dictionary read through L1:
-// for dictionaries too large for zf_strdict_sm.cu, and in batched launches.
+// for dictionaries too large for zf_strdict_sm.cu, for launches of many chunks
+// of few tiles, and in batched launches.
 #pragma once
 #include "zf_device.cuh"
 

@@ -1,7 +1,8 @@
 """String-dictionary decode around the sizes where the shared-memory kernel's
 batches (64 tokens), tiles (1024 tokens), dictionaries and CTA ranges begin and
-end, and columns whose chunks take both kernels (dictionaries that fit in
-shared memory and ones that do not)."""
+end, columns whose chunks take both kernels (dictionaries that fit in shared
+memory and ones that do not), and short chunks on either side of the four per
+SM (608 on 152 SMs) from which a launch reads them through L1."""
 import numpy as np
 import pytest
 
@@ -34,6 +35,8 @@ CASES = {
     "every length": lambda: (_text(9, _words(9, 900, 1, 64), 30_000), 131072),
     "single bytes": lambda: (np.random.default_rng(10).integers(0, 256, 200_003).astype(np.uint8), 65536),
     "1,025 entries": lambda: (_text(11, _words(11, 1025, 6, 8), 40_000), 1 << 20),
+    "few short chunks": lambda: (_text(17, _words(17, 900, 3, 12), 4_500_000), 65536),
+    "many short chunks": lambda: (_text(18, _words(18, 900, 3, 12), 6_500_000), 65536),
     "CTA ranges across many chunks": lambda: (_text(12, _words(12, 3000, 3, 12), 900_000), 65536),
     "one chunk over all CTAs": lambda: (_text(13, _words(13, 5000, 3, 12), 500_000), 1 << 23),
     "dictionaries at the shared-memory limit": lambda: (_text(14, _words(14, 13_000, 6, 9), 300_000), 1 << 19),
