@@ -313,8 +313,10 @@ typedef struct {
  * 32, 64; for string columns the class of their bytes, the offsets being a
  * small second part) -- the result is kept for that class: later launches of the class
  * use it while the context's tile_rows / threads are 0 (automatic), so one
- * tuning run per column kind gives every kind its own geometry.  Otherwise
- * the result becomes the context's geometry.  A resident search of one
+ * tuning run per column kind gives every kind its own geometry.  Where no
+ * launch of the columns takes a geometry (zf_kcfg.tile_rows), none is kept:
+ * every point was the same launch.  Columns of several classes: the result
+ * becomes the context's geometry.  A resident search of one
  * class also records the class's decode rate at the fastest point (plain
  * bytes / time), which Johnson's rule then uses.  Outputs as in
  * zf_transfer_decompress; the columns are decoded into them many times. */
@@ -333,14 +335,18 @@ zf_status zf_tune(zf_ctx* ctx, const zf_compressed* const* cols, uint32_t ncols,
 zf_status zf_tune_chunk_rows(zf_ctx* ctx, const zf_column* col, int32_t scheme, const uint32_t* chunk_rows,
                              uint32_t n, uint32_t reps, float* ms, uint32_t* best);
 
-/* The geometry a launch of one class would use now: the context's
+/* The geometry a large launch of one class would use now: the context's
  * tile_rows / threads where set, else the class's tuned entry, else the
  * built-in values (128 threads; warp jobs of 2048 rows for delta, 4096 for
- * the others).  bmax = the widest bit width of the launch's chunks. */
+ * the others, which launches of few rows halve: zf_kcfg.tile_rows, where the
+ * kernels that take no geometry stand too).  bmax = the widest bit width of
+ * the launch's chunks. */
 zf_status zf_ctx_tuned_geometry(const zf_ctx* ctx, int32_t scheme, int32_t dtype, uint32_t bmax, zf_kcfg* out);
 
 /* The measured rates Johnson's rule reads for a class: the decode rate a
- * resident zf_tune of that class recorded (plain GB/s) and the link rate the
+ * resident zf_tune of that class recorded (plain GB/s; string dictionaries
+ * that fit in shared memory and larger ones are kept apart, and the former's
+ * is given where there is one) and the link rate the
  * last zf_measure_copy recorded (compressed GB/s); 0 where none was measured
  * (the ordering then uses nominal rates).  Either pointer may be NULL. */
 zf_status zf_ctx_rates(const zf_ctx* ctx, int32_t scheme, int32_t dtype, uint32_t bmax, float* decode_gbs,

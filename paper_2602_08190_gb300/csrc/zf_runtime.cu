@@ -72,6 +72,8 @@ struct zf_ctx {
         uint32_t tile_rows = 0, threads = 0;
         float gbs = 0;                 // measured decode rate at that geometry (plain GB/s), 0 = none
     } tuned[ZF_NSCHEMES][4][4];
+    float strdict_shared_gbs[4] = {0}; // the rate of string dictionaries held in shared memory, per bit-width bucket
+    uint64_t tile_launches[ZF_NSCHEMES + 1] = {0};   // launches that take a geometry, per scheme; last: batched ones
     float link_gbs = 0;               // measured host-to-device rate of the call's pieces (zf_measure_copy), 0 = none
     uint64_t tuned_gen = 0;
     uint64_t slots_gen = 0;        // bumped whenever the staging slots are reallocated
@@ -367,6 +369,7 @@ zf_status launch_groups(zf_ctx* ctx, const Group* groups, size_t ngroups, const 
             zf::TileLaunch L{dchunks, hchunks, g.count, g.ntiles, g.scheme, g.dtype, g.tile_rows, g.threads,
                              k.ctas_per_sm, smem, ctx->num_sms, ctx->d_errw, queue};
             e = zf::launch_tiles(L, stream);
+            ctx->tile_launches[g.scheme < 0 ? ZF_NSCHEMES : g.scheme]++;
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "decode launch");
         ctx->st.n_launches++;
@@ -407,7 +410,9 @@ void johnson_order(const zf_ctx* ctx, std::vector<Work>& work) {
             const zf::ChunkInfo& c = *work[j].ch;
             const double plain = (double)c.rows * zf::dtype_size(c.dtype);
             double rate = 0;
-            if (c.scheme < ZF_NSCHEMES && c.dtype < 4) rate = ctx->tuned[c.scheme][c.dtype][width_bucket(c.bmax)].gbs;
+            if (fits_shared(c)) rate = ctx->strdict_shared_gbs[width_bucket(c.bmax)];
+            if (!(rate > 0) && c.scheme < ZF_NSCHEMES && c.dtype < 4)
+                rate = ctx->tuned[c.scheme][c.dtype][width_bucket(c.bmax)].gbs;
             if (!(rate > 0)) rate = nominal_decode_gbs(c.scheme);
             cp += (double)c.bytes / link;
             dc += plain / rate;
@@ -1279,6 +1284,8 @@ extern "C" zf_status zf_tune(zf_ctx* ctx, const zf_compressed* const* cols, uint
     uint32_t n = 0;
     float best_ms = 3.0e38f;
     zf_kcfg best_k = saved;
+    uint64_t launches[ZF_NSCHEMES + 1];   // before the search
+    std::copy(std::begin(ctx->tile_launches), std::end(ctx->tile_launches), launches);
     for (uint32_t gi = 0; gi < ngraph; gi++)
     for (uint32_t si = 0; si < nstage; si++)
         for (uint32_t tr : kTuneTileRows)
@@ -1334,12 +1341,18 @@ extern "C" zf_status zf_tune(zf_ctx* ctx, const zf_compressed* const* cols, uint
             cb = b;
         }
     if (one && cs >= 0) {
-        ctx->tuned[cs][cd][cb].tile_rows = best_k.tile_rows;
-        ctx->tuned[cs][cd][cb].threads = best_k.threads;
+        // kernels with fixed jobs (LZ77, ANS, string dictionaries in shared memory) make every point the same launch:
+        // the fastest is chance, and the larger dictionaries of a width class do take its geometry
+        const bool geometry = ctx->tile_launches[cs] != launches[cs] || ctx->tile_launches[ZF_NSCHEMES] != launches[ZF_NSCHEMES];
+        if (geometry) {
+            ctx->tuned[cs][cd][cb].tile_rows = best_k.tile_rows;
+            ctx->tuned[cs][cd][cb].threads = best_k.threads;
+        }
         if (!transfer && best_ms > 0) {
             uint64_t raw = 0;
             for (uint32_t c = 0; c < ncols; c++) raw += cols[c]->raw_bytes;
-            ctx->tuned[cs][cd][cb].gbs = (float)((double)raw / (best_ms * 1e6));
+            (cs == ZF_STRDICT && !geometry ? ctx->strdict_shared_gbs[cb] : ctx->tuned[cs][cd][cb].gbs) =
+                (float)((double)raw / (best_ms * 1e6));
         }
         ctx->tuned_gen++;
         ctx->kcfg = saved;
@@ -1358,7 +1371,11 @@ extern "C" zf_status zf_tune(zf_ctx* ctx, const zf_compressed* const* cols, uint
 extern "C" zf_status zf_ctx_rates(const zf_ctx* ctx, int32_t scheme, int32_t dtype, uint32_t bmax, float* decode_gbs,
                                   float* link_gbs) {
     if (!ctx || scheme < 0 || scheme >= ZF_NSCHEMES || dtype < 0 || dtype > ZF_F64 || bmax > 64) return ZF_EINVAL;
-    if (decode_gbs) decode_gbs[0] = ctx->tuned[scheme][dtype][width_bucket(bmax)].gbs;
+    if (decode_gbs) {
+        decode_gbs[0] = ctx->tuned[scheme][dtype][width_bucket(bmax)].gbs;
+        if (scheme == ZF_STRDICT && dtype == ZF_BYTES && ctx->strdict_shared_gbs[width_bucket(bmax)] > 0)
+            decode_gbs[0] = ctx->strdict_shared_gbs[width_bucket(bmax)];
+    }
     if (link_gbs) link_gbs[0] = ctx->link_gbs;
     return ZF_OK;
 }

@@ -159,3 +159,44 @@ def test_tune_chunk_rows_times_every_candidate(columns):
             zf.zf_compressed_free(h)
     finally:
         g.close()
+
+
+def test_tune_keeps_no_geometry_of_a_kernel_that_takes_none():
+    """Every point of a search over a string dictionary in shared memory (and
+    over LZ77 and ANS) is the same launch: the fastest is chance, and larger
+    dictionaries of the same width class would take it over.  The rate stays."""
+    def text(words, n):
+        r = np.random.default_rng(words)
+        w = [b"w%06d " % i for i in range(words)]
+        return np.frombuffer(b"".join(w[i] for i in r.integers(0, words, n)), np.uint8).copy()
+
+    small, large = text(5_000, 150_000), text(40_000, 150_000)     # 13 and 16 bits: one class
+    flags = np.random.default_rng(1).integers(0, 3, 200_000).astype(np.int32)
+    g = Gpu()
+    try:
+        def tune(x, scheme, chunk_rows, resident=True):
+            o = np.array([0, len(x)], np.int32) if x.dtype == np.uint8 else None
+            col = zf.Column(x, o)
+            h = zf.zf_compress_host(zf.zf_plan(None, col, scheme=scheme, chunk_rows=chunk_rows), col)
+            bufs = g.alloc(out_specs(x, o))
+            pts, best = zf.zf_tune(g.ctx, [h], [b.data_ptr() for b in bufs], [b.numel() for b in bufs], transfer=not resident, reps=1)
+            assert np.array_equal(bufs[0].cpu().numpy()[:x.nbytes].view(x.dtype), x)
+            zf.zf_compressed_free(h)
+            return best
+
+        def geometry(scheme, dtype, bits):
+            k = zf.zf_ctx_tuned_geometry(g.ctx, scheme, dtype, bits)
+            return k.tile_rows, k.threads
+
+        for x, scheme, chunk, dtype, bits in [(small, zf.ZF_STRDICT, 1 << 20, zf.ZF_BYTES, 13), (small, zf.ZF_LZ77, 0, zf.ZF_BYTES, 0),
+                                              (flags, zf.ZF_ANS, 65536, zf.ZF_I32, 0)]:
+            for resident in (True, False):
+                tune(x, scheme, chunk, resident)
+                assert geometry(scheme, dtype, bits) == (4096, 128)
+            assert zf.zf_ctx_rates(g.ctx, scheme, dtype, bits)[0] > 0
+        shared = zf.zf_ctx_rates(g.ctx, zf.ZF_STRDICT, zf.ZF_BYTES, 13)[0]
+        best = tune(large, zf.ZF_STRDICT, 1 << 21)
+        assert geometry(zf.ZF_STRDICT, zf.ZF_BYTES, 16) == (best.tile_rows, best.threads)
+        assert zf.zf_ctx_rates(g.ctx, zf.ZF_STRDICT, zf.ZF_BYTES, 16)[0] == shared
+    finally:
+        g.close()
