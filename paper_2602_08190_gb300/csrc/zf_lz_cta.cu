@@ -309,7 +309,10 @@ __device__ void lz_block(const ZfDevChunk& c, LzSmem& sm, uint32_t* err) {
                     const uint2* u = &sm.tok[n ? n - 1 : 0];
                     const uint32_t ux = *const_cast<const volatile uint32_t*>(&u->x);   // its owner may shorten it meanwhile
                     if (src <= (ux & 0xFFFFu) || src + ml - 1 > (u->y >> 16)) break;
-                    o += ux >> 16;
+                    // a match that overlaps its own output (a run): into its first period at once, not period by period
+                    const uint32_t uo = ux >> 16, d = src - 1 - (ux & 0xFFFFu);
+                    o += uo;
+                    if (d >= uo) o += d / uo * uo;
                     *reinterpret_cast<volatile uint32_t*>(&sm.tok[tid].x) = (mpos - 1) | (o << 16);
                 }
             }

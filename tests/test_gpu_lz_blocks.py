@@ -64,6 +64,10 @@ CASES = {
     "1,025 tokens of 16 literals": (1025, (16, 16), (4, 40), FAR, False),
     "16,384 shortest tokens": (16384, (0, 0), (4, 4), NEAR, False),
     "long literal runs": (8, (7000, 8200), (4, 9), FAR, True),
+    "512 tokens of 60 literals": (512, (60, 60), (4, 9), NEAR, False),
+    "some 20 literals a token, padded": (1500, (10, 33), (4, 9), FAR, True),
+    "some 150 literals a token": (300, (100, 205), (4, 20), FAR, False),
+    "literal runs of a page and matches of one": (14, (2000, 2600), (2000, 2100), NEAR, False),
     "long matches": (12, (1, 2), (5000, 5400), FAR, False),
 }
 
@@ -118,3 +122,47 @@ def test_hand_made_blocks_in_a_large_launch():
         g.close()
         for h in handles:
             zf.zf_compressed_free(h)
+
+
+# Contents beyond text: a run that copies a run's end (its source lies in a
+# match that overlaps its own output), runs after literals, periods, and
+# blocks with more literals than a batch's ring, in launches of one block, of
+# few and of many per SM.
+def _runs(r, n):
+    x = r.integers(0, 256, n).astype(np.uint8)
+    x[(np.arange(n) // 512) % 2 == 0] = 0
+    return x
+
+
+def _padded(r, n):
+    x = r.integers(0, 256, n).astype(np.uint8)
+    x[(np.arange(n) % 100) < 60] = 32
+    return x
+
+
+CONTENTS = {
+    "runs between literals": _runs,
+    "padded fields": _padded,
+    "long periods": lambda r, n: np.where(r.random(n) < 0.0003, r.integers(0, 256, n), np.resize(r.integers(0, 256, 37), n)).astype(np.uint8),
+    "short runs": lambda r, n: np.repeat(r.integers(0, 3, n // 20 + 2), r.integers(1, 60, n // 20 + 2))[:n].astype(np.uint8),
+    "zeros": lambda r, n: np.zeros(n, np.uint8),
+}
+
+
+@pytest.mark.parametrize("blocks", [1, 40, 1500, 2000])
+@pytest.mark.parametrize("name", CONTENTS)
+def test_contents(name, blocks):
+    from gpu_helpers import Gpu
+    n = blocks * 65536 - 77
+    t = CONTENTS[name](np.random.default_rng(blocks), n)
+    assert len(t) == n
+    o = np.array([0, n], np.int32)
+    col = zf.Column(t, o)
+    h = zf.zf_compress_host(zf.zf_plan(None, col, scheme=zf.ZF_LZ77), col)
+    g = Gpu()
+    try:
+        got, _ = g.decode([h], [(np.uint8, n), (np.int32, 2)], resident=True)
+        assert np.array_equal(got, t)
+    finally:
+        zf.zf_compressed_free(h)
+        g.close()
