@@ -123,13 +123,16 @@ __device__ __forceinline__ uint2 lz_lookup(const LzSmem& sm, const uint8_t* __re
             v[b] = here ? (uint32_t)m + b - base : kDone | x;
         }
         if (over) {
+            uint32_t rem = j0 > la ? (j0 - la - 1) % oa : 0u;   // byte 0's place in the match's period; the next ones' follow
 #pragma unroll
             for (uint32_t b = 0; b < 4; b++) {
                 const bool second = b >= pb;
                 const uint32_t last = second ? lb : la, off = second ? ob : oa, j = j0 + b;
-                if (j <= last || j - off <= last || j < s0 || j >= s1) continue;
-                const uint32_t src = last + 1 - off + (j - last - 1) % off;
-                v[b] = src >= s0 ? src - base : kDone | sm.out[src];
+                if (b == pb) rem = 0;
+                if (j <= last) continue;
+                const uint32_t src = last + 1 - off + rem;
+                rem = rem + 1 == off ? 0 : rem + 1;
+                if (j >= s0 && j < s1) v[b] = src >= s0 ? src - base : kDone | sm.out[src];
             }
         }
         if (j0 < s0 || j0 + 4 > s1) {   // bytes outside the segment: nothing copies them
