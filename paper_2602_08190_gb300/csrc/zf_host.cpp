@@ -1073,6 +1073,10 @@ zf_status parse_serialized(zf_compressed* c, std::string* why) {
             expect += ch.bytes;
             if (!check_chunk(h + ch.off, ch.bytes, pi.scheme, pi.dtype, ch.rows, &ch.bmax, why)) return ZF_ECORRUPT;
             if (pi.scheme == ZF_STRDICT || pi.scheme == ZF_ANS) ch.units = (uint32_t)rd<uint64_t>(h + ch.off + 16);
+            if (pi.scheme == ZF_LZ77 && !(h[ch.off + 7] & 1)) {
+                const uint64_t tokens = rd<uint32_t>(h + ch.off + 12), lits = rd<uint32_t>(h + ch.off + 44);
+                ch.lz_runs = lits > 16 * tokens && lits + 16 * tokens < ch.rows;
+            }
             if (pi.scheme == ZF_STRDICT) ch.dict_bytes = rd<uint32_t>(h + ch.off + 40) + 7u * rd<uint32_t>(h + ch.off + 12);
             ch.off += pos;
             ch.scheme = (uint8_t)pi.scheme;

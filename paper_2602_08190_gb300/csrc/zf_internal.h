@@ -70,6 +70,7 @@ struct ChunkInfo {
     uint8_t scheme, dtype, part;
     uint8_t bmax;     // widest bit width in the chunk (FOR/DICT: b; DELTA: widest block)
     uint32_t units = 0;   // string dictionary: tokens of the chunk; ANS: streams
+    bool lz_runs = false; // LZ77: on average more than 16 literals and 16 copied bytes to a token
     uint32_t dict_bytes = 0;  // string dictionary: most shared memory its dictionary takes (a word per entry, entries padded to words)
 };
 

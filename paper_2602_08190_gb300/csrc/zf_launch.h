@@ -54,7 +54,9 @@ struct TileLaunch {
 
 uint32_t warp_smem_bytes(int scheme, int dtype, uint32_t bmax);
 cudaError_t launch_tiles(const TileLaunch& L, cudaStream_t s);
-cudaError_t launch_lz(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t n, uint32_t* err, int num_sms, cudaStream_t s);
+// LZ77 blocks, `runs` of them with ChunkInfo::lz_runs.
+cudaError_t launch_lz(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t n, uint32_t runs, uint32_t* err,
+                      int num_sms, cudaStream_t s);
 cudaError_t launch_lz_cta(const ChunkArgs& chunks, uint32_t* err, cudaStream_t s);
 // String-dictionary chunks whose dictionaries take at most dict_bytes
 // (ChunkInfo::dict_bytes, at most strdict_smem_limit()) of shared memory;

@@ -44,7 +44,11 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 // are, a CTA per block adds 0.3 us for each block to about 60 us: resident
 // calls of 16, 64 and 128 MB took 118, 368 and 683 us with a CTA and 578, 681
 // and 785 us with a warp per block; 160 MB, 17 blocks per SM, would be even.
-constexpr uint32_t kLzCtaBlocksPerSm = 15;
+// Blocks of long literal runs between long matches (fields padded with blanks)
+// leave the warp kernel little to parse and the CTA kernel literals that its
+// ring does not hold: 64 and 130 MB took 331 and 605 us with a CTA, 414 and 495
+// with a warp per block, so where most blocks are such the line is at 9 per SM.
+constexpr uint32_t kLzCtaBlocksPerSm = 15, kLzCtaRunBlocksPerSm = 9;
 
 struct LzParse {
     uint32_t vp = 0;        // next byte of the lengths stream
@@ -336,10 +340,11 @@ __global__ void __launch_bounds__(32, 32) lz_kernel(const ZfDevChunk* chunks, ui
 
 namespace zf {
 
-cudaError_t launch_lz(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t n, uint32_t* err, int num_sms,
-                      cudaStream_t s) {
+cudaError_t launch_lz(const ZfDevChunk* chunks, const ZfDevChunk* host, uint32_t n, uint32_t runs, uint32_t* err,
+                      int num_sms, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    if (n <= (uint32_t)num_sms * kLzCtaBlocksPerSm || !chunks) return launch_lz_cta(ChunkArgs(chunks, host, n), err, s);
+    const uint32_t per_sm = runs > n / 2 ? kLzCtaRunBlocksPerSm : kLzCtaBlocksPerSm;
+    if (n <= (uint32_t)num_sms * per_sm || !chunks) return launch_lz_cta(ChunkArgs(chunks, host, n), err, s);
     // one warp (one block) per CTA, so a small launch still spreads over
     // every SM; up to 32 CTAs per SM, then warps loop over the rest
     uint32_t blocks = n;

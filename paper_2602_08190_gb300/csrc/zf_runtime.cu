@@ -250,6 +250,7 @@ struct Group {
     uint32_t tile_rows;  // rows of a warp job in this launch
     uint32_t threads;    // threads per CTA of this launch
     uint32_t dict_bytes; // kStrdictSmem: most shared memory a chunk's dictionary takes
+    uint32_t lz_runs;    // LZ77: chunks with ChunkInfo::lz_runs
 };
 
 // Group::scheme of string-dictionary chunks whose dictionary fits in shared
@@ -298,7 +299,7 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         std::pair<int, int> key;
         uint32_t bmax = 0;         // widest bit width of the group: its geometry class
         uint64_t units = 0;        // rows (string dictionary: tokens) of the group
-        uint32_t dict_bytes = 0;
+        uint32_t dict_bytes = 0, lz_runs = 0;
     };
     std::vector<Key> keys;
     std::vector<uint8_t> key_of(e - b);   // a call has few groups: at most one per scheme and type
@@ -312,13 +313,15 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         if (key.first >= 0) keys[q].bmax = std::max<uint32_t>(keys[q].bmax, ch.bmax);
         keys[q].units += ch.scheme == ZF_STRDICT ? ch.units : ch.rows;
         keys[q].dict_bytes = std::max(keys[q].dict_bytes, ch.dict_bytes);
+        keys[q].lz_runs += ch.lz_runs;
     }
     for (size_t q = 0; q < keys.size(); q++) {
         const Key& kq = keys[q];
         const auto& key = kq.key;
         const Geometry geo = key.first == kStrdictSmem ? Geometry{zf::kStrTile, 0}
                                                        : group_geometry(ctx, k, key.first, key.second, kq.bmax, kq.units);
-        Group g{key.first, key.second, (uint32_t)desc.size(), 0, 0, 16, geo.tile_rows, geo.threads, kq.dict_bytes};
+        Group g{key.first, key.second, (uint32_t)desc.size(), 0, 0, 16, geo.tile_rows, geo.threads, kq.dict_bytes,
+                kq.lz_runs};
         for (size_t i = b; i < e; i++) {
             if (key_of[i - b] != q) continue;
             const int s = w[i].ch->scheme, d = w[i].ch->dtype;
@@ -359,7 +362,7 @@ zf_status launch_groups(zf_ctx* ctx, const Group* groups, size_t ngroups, const 
         const ZfDevChunk *dchunks = d_desc ? d_desc + g.first : nullptr, *hchunks = h_desc + g.first;
         cudaError_t e;
         if (g.scheme == ZF_LZ77) {
-            e = zf::launch_lz(dchunks, hchunks, g.count, ctx->d_errw, ctx->num_sms, stream);
+            e = zf::launch_lz(dchunks, hchunks, g.count, g.lz_runs, ctx->d_errw, ctx->num_sms, stream);
         } else if (g.scheme == kStrdictSmem) {
             e = zf::launch_strdict(dchunks, hchunks, g.count, g.ntiles, g.dict_bytes, ctx->d_errw, ctx->num_sms, stream);
         } else if (g.scheme == ZF_ANS) {
