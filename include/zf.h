@@ -144,7 +144,9 @@ typedef struct {
     uint32_t tile_rows;       /* rows per warp job: a multiple of 1024, <= 16384 (0 = the
                                  class's tuned value, else 2048 for delta launches
                                  and 4096 for the others, halved down to 1024 while
-                                 a launch has fewer than 32 jobs per SM); LZ77, ANS and
+                                 a launch has fewer than 32 jobs per SM; FOR and
+                                 dictionary launches: 1024 below 8 and 14, 2048 while
+                                 more than run at once but fewer than 32); LZ77, ANS and
                                  string dictionaries that fit in shared memory (without
                                  ZF_KCFG_BATCHED; not launches of many chunks of under
                                  16,384 tokens) have fixed jobs and read neither this

@@ -45,6 +45,7 @@ struct zf_resident {
 struct zf_ctx {
     int device = 0;
     int num_sms = 0;
+    uint32_t smem_per_sm = 0;      // bytes of shared memory
     cudaStream_t copy = nullptr, compute = nullptr;
     cudaStream_t lane[kMaxSlots] = {};  // decode stream of each staging slot
     bool own_copy = false, own_compute = false;
@@ -126,24 +127,42 @@ uint32_t width_bucket(uint32_t bmax) { return bmax <= 8 ? 0u : bmax <= 16 ? 1u :
 struct Geometry {
     uint32_t tile_rows, threads;
 };
-// The built-in job is halved while the launch's `units` (rows or tokens) would
-// give an SM fewer than 32 warps: a job's tiles follow one another, so in a
-// launch that leaves warps idle every tile but the first only waits (a
-// resident call of 1M rows took 24.4, 30.4 and 38.1 us as FOR, RLE and
-// Float2Int and takes 22.6, 23.6 and 25.6 us; 4 MB of string dictionary 107
-// and 71 us; from 32M rows on nothing changes).  units = 0: not known.
-Geometry group_geometry(const zf_ctx* ctx, const zf_kcfg& k, int scheme, int dtype, uint32_t bmax, uint64_t units) {
+// The built-in job of a launch of few `units` (rows or tokens; 0: not known).
+// A job's tiles follow one another, so in a launch that leaves warps idle
+// every tile but the first only waits: the job is halved while an SM would get
+// fewer than 32 warps (a resident call of 1M rows took 24.4, 30.4 and 38.1 us
+// as FOR, RLE and Float2Int and takes 22.6, 23.6 and 25.6; 4 MB of string
+// dictionary 107 and 71; from 32M rows on nothing changes).  FOR and
+// dictionary tiles are short beside a job's own start (its chunk, the header,
+// the first bytes), so their jobs stay whole from 8 (FOR) or 14 warps per SM
+// on, except that more than run at once, up to 32, are halved for the second
+// wave's sake.  Device time of FOR in 64K-row chunks, halved down to 1,024 rows
+// and now: 6.5M rows of 62 bits 24.7 and 18.7 us, of 40 bits 18.4 and 16.4, of
+// 24 bits 12.4 and 12.2; 17M rows of 40 bits 49.5 whole and 44.8 halved once; of
+// 1,000 int64 values 47.2 halved once and 41.3.  (Batched launches that hold
+// other schemes too are halved: a fact table of 16 columns of 0.7M rows, two
+// thirds of them FOR and dictionaries, takes 43 us, 48 with whole jobs.)
+Geometry group_geometry(const zf_ctx* ctx, const zf_kcfg& k, int scheme, int dtype, uint32_t bmax, uint64_t units,
+                        uint64_t short_tiled) {
     Geometry g{k.tile_rows, k.threads};
     if (scheme >= 0 && scheme < ZF_NSCHEMES && dtype >= 0 && dtype < 4) {
         const auto& t = ctx->tuned[scheme][dtype][width_bucket(bmax)];
         if (!g.tile_rows) g.tile_rows = t.tile_rows;
         if (!g.threads) g.threads = t.threads;
     }
-    if (!g.tile_rows) {
-        g.tile_rows = scheme == ZF_DELTA_BP ? 2048u : 4096u;
-        while (units && g.tile_rows > 1024 && units < (uint64_t)g.tile_rows * 32u * ctx->num_sms) g.tile_rows /= 2;
-    }
     if (!g.threads) g.threads = 128;
+    if (g.tile_rows) return g;
+    g.tile_rows = scheme == ZF_DELTA_BP ? 2048u : 4096u;
+    const uint64_t per_sm = units / std::max(1, ctx->num_sms);
+    if (units && short_tiled == units) {
+        const uint32_t few = scheme == ZF_DICT_BP ? 14 : 8;
+        const uint32_t cta = (scheme < 0 ? 0 : zf::warp_smem_bytes(scheme, dtype, bmax)) * (g.threads / 32) + 1024;
+        const uint32_t at_once = std::min(32u, ctx->smem_per_sm / cta * (g.threads / 32));   // warps of an SM
+        if (per_sm < 4096ull * few) g.tile_rows = 1024;
+        else if (per_sm > 4096ull * at_once && per_sm < 4096ull * 32) g.tile_rows = 2048;
+        return g;
+    }
+    while (units && g.tile_rows > 1024 && per_sm < (uint64_t)g.tile_rows * 32) g.tile_rows /= 2;
     return g;
 }
 
@@ -299,6 +318,7 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         std::pair<int, int> key;
         uint32_t bmax = 0;         // widest bit width of the group: its geometry class
         uint64_t units = 0;        // rows (string dictionary: tokens) of the group
+        uint64_t short_tiled = 0;  // those of FOR and dictionary chunks
         uint32_t dict_bytes = 0, lz_runs = 0;
     };
     std::vector<Key> keys;
@@ -312,6 +332,7 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         key_of[i - b] = (uint8_t)q;
         if (key.first >= 0) keys[q].bmax = std::max<uint32_t>(keys[q].bmax, ch.bmax);
         keys[q].units += ch.scheme == ZF_STRDICT ? ch.units : ch.rows;
+        if (ch.scheme == ZF_FOR_BP || ch.scheme == ZF_DICT_BP) keys[q].short_tiled += ch.rows;
         keys[q].dict_bytes = std::max(keys[q].dict_bytes, ch.dict_bytes);
         keys[q].lz_runs += ch.lz_runs;
     }
@@ -319,7 +340,8 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         const Key& kq = keys[q];
         const auto& key = kq.key;
         const Geometry geo = key.first == kStrdictSmem ? Geometry{zf::kStrTile, 0}
-                                                       : group_geometry(ctx, k, key.first, key.second, kq.bmax, kq.units);
+                                                       : group_geometry(ctx, k, key.first, key.second, kq.bmax, kq.units,
+                                                                        kq.short_tiled);
         Group g{key.first, key.second, (uint32_t)desc.size(), 0, 0, 16, geo.tile_rows, geo.threads, kq.dict_bytes,
                 kq.lz_runs};
         for (size_t i = b; i < e; i++) {
@@ -530,6 +552,9 @@ zf_status zf_ctx_create(int device, void* copy_stream, void* compute_stream, zf_
     };
     if (cudaSetDevice(device) != cudaSuccess) return fail(ZF_ECUDA);
     cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
+    int smem = 0;
+    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
+    ctx->smem_per_sm = (uint32_t)smem;
     if (copy_stream) ctx->copy = (cudaStream_t)copy_stream;
     else if (cudaStreamCreateWithFlags(&ctx->copy, cudaStreamNonBlocking) == cudaSuccess) ctx->own_copy = true;
     else return fail(ZF_ECUDA);
@@ -1388,7 +1413,7 @@ extern "C" zf_status zf_ctx_tuned_geometry(const zf_ctx* ctx, int32_t scheme, in
     if (!ctx || !out || scheme < 0 || scheme >= ZF_NSCHEMES || dtype < 0 || dtype > ZF_F64 || bmax > 64)
         return ZF_EINVAL;
     const zf_kcfg k = effective_kcfg(ctx);
-    const Geometry g = group_geometry(ctx, k, scheme, dtype, bmax, 0);
+    const Geometry g = group_geometry(ctx, k, scheme, dtype, bmax, 0, 0);
     *out = k;
     out->tile_rows = g.tile_rows;
     out->threads = g.threads;
