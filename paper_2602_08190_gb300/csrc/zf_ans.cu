@@ -158,14 +158,24 @@ __device__ __forceinline__ void ans_ask(AnsSmem& sm, const uint8_t* s2, uint32_t
     __pipeline_commit();
 }
 
-// Slot entries: warp w fills the ranges of symbols w, w + kWarps, ..., a range's
-// slots side by side over the lanes.  (A contiguous 32 slots per thread, each
-// thread walking its symbols, took 4 to 8 us more of a call.)
+// Slot entries: warp w fills the ranges of symbols w, w + kWarps, ... (lane l has
+// every 32nd of them): a range of up to kShort slots by its lane, a longer one by
+// the whole warp, its slots side by side over the lanes.  (A contiguous 32 slots
+// per thread, each thread walking its symbols, took 4 to 8 us more of a call of
+// few symbols; all ranges by whole warps 4 us more of one of 256.)
 template <bool WIDE>
 __device__ __forceinline__ void ans_table(AnsSmem& sm, uint32_t nd, uint32_t lane, uint32_t warp) {
-    for (uint32_t s = warp; s < nd; s += kWarps) {
-        const uint32_t c = sm.cum[s], f = sm.cum[s + 1] - c;
-        for (uint32_t d = lane; d < f; d += 32) sm.slot[c + d] = ans_entry<WIDE>(s, f, d);
+    constexpr uint32_t kShort = 16;
+    for (uint32_t s0 = warp; s0 < nd; s0 += 32 * kWarps) {
+        const uint32_t s = s0 + lane * kWarps;
+        const uint32_t c = s < nd ? sm.cum[s] : 0u, f = s < nd ? sm.cum[s + 1] - c : 0u;
+        if (f <= kShort)
+            for (uint32_t d = 0; d < f; d++) sm.slot[c + d] = ans_entry<WIDE>(s, f, d);
+        for (uint32_t m = __ballot_sync(0xFFFFFFFFu, f > kShort); m; m &= m - 1) {
+            const uint32_t l = __ffs(m) - 1;
+            const uint32_t ck = __shfl_sync(0xFFFFFFFFu, c, l), fk = __shfl_sync(0xFFFFFFFFu, f, l);
+            for (uint32_t d = lane; d < fk; d += 32) sm.slot[ck + d] = ans_entry<WIDE>(s0 + l * kWarps, fk, d);
+        }
     }
 }
 
