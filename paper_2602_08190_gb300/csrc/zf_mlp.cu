@@ -61,19 +61,33 @@ __device__ __forceinline__ uint32_t row_of(const Rows& r, uint32_t i) { return r
 __device__ __forceinline__ void forward_tile(const float* __restrict__ p, const Rows& r, MlpSmem& sm) {
     const int tid = threadIdx.x;
     const uint32_t s0 = blockIdx.x * kTile;
-    for (int i = tid; i < HID * IN; i += kThreads) sm.w1[i / IN * (IN + 1) + i % IN] = p[OW1 + i];
-    for (int i = tid; i < HID * HID; i += kThreads) sm.w2[i / HID * (HID + 1) + i % HID] = p[OW2 + i];
-    for (int i = tid; i < OUT * HID; i += kThreads) sm.w3[i / HID * (HID + 1) + i % HID] = p[OW3 + i];
-    if (tid < HID) sm.b1[tid] = p[OB1 + tid];
-    else if (tid < 2 * HID) sm.b2[tid - HID] = p[OB2 + tid - HID];
-    else if (tid < 2 * HID + OUT) sm.b3[tid - 2 * HID] = p[OB3 + tid - 2 * HID];
-    {
-        static_assert(kThreads == IN * kTile, "one input value per thread");
-        const int s = tid / IN, i = tid % IN;
-        float v = s0 + s < r.n ? r.X[(size_t)row_of(r, s0 + s) * IN + i] : 0.0f;
-        if (r.scaled) v = (v - r.mean[i]) / r.sd[i];
-        sm.x[i * kTile + s] = v;
-    }
+    // every load is under way before the first value is stored: a thread's 28 weights, a bias and an input value
+    // one after another held up a batch of up to 64 samples by 2 us
+    static_assert(kThreads == IN * kTile, "one input value per thread");
+    const int s = tid / IN, f = tid % IN;
+    float x = s0 + s < r.n ? r.X[(size_t)row_of(r, s0 + s) * IN + f] : 0.0f;
+    constexpr int N1 = HID * IN / kThreads, N2 = HID * HID / kThreads, N3 = OUT * HID / kThreads;
+    float w1[N1], w2[N2], w3[N3], b = 0.0f;
+#pragma unroll
+    for (int q = 0; q < N1; q++) w1[q] = p[OW1 + tid + q * kThreads];
+#pragma unroll
+    for (int q = 0; q < N2; q++) w2[q] = p[OW2 + tid + q * kThreads];
+#pragma unroll
+    for (int q = 0; q < N3; q++) w3[q] = p[OW3 + tid + q * kThreads];
+    if (tid < HID) b = p[OB1 + tid];
+    else if (tid < 2 * HID) b = p[OB2 + tid - HID];
+    else if (tid < 2 * HID + OUT) b = p[OB3 + tid - 2 * HID];
+#pragma unroll
+    for (int q = 0; q < N1; q++) sm.w1[(tid + q * kThreads) / IN * (IN + 1) + (tid + q * kThreads) % IN] = w1[q];
+#pragma unroll
+    for (int q = 0; q < N2; q++) sm.w2[(tid + q * kThreads) / HID * (HID + 1) + (tid + q * kThreads) % HID] = w2[q];
+#pragma unroll
+    for (int q = 0; q < N3; q++) sm.w3[(tid + q * kThreads) / HID * (HID + 1) + (tid + q * kThreads) % HID] = w3[q];
+    if (tid < HID) sm.b1[tid] = b;
+    else if (tid < 2 * HID) sm.b2[tid - HID] = b;
+    else if (tid < 2 * HID + OUT) sm.b3[tid - 2 * HID] = b;
+    if (r.scaled) x = (x - r.mean[f]) / r.sd[f];
+    sm.x[f * kTile + s] = x;
     __syncthreads();
     const int j = tid & (HID - 1), g = tid / HID * 2;
     {
