@@ -407,11 +407,11 @@ zf_status launch_groups(zf_ctx* ctx, const Group* groups, size_t ngroups, const 
 double nominal_decode_gbs(int scheme) {
     switch (scheme) {
     case ZF_LZ77: return 300;
-    case ZF_RLE: return 3500;
+    case ZF_RLE: return 4200;
     case ZF_DELTA_BP: case ZF_DICT_BP: return 5000;
-    case ZF_FLOAT2INT: return 1500;
-    case ZF_STRDICT: return 1000;
-    case ZF_ANS: return 500;
+    case ZF_FLOAT2INT: return 4200;
+    case ZF_STRDICT: return 1400;   // in shared memory; larger dictionaries 850
+    case ZF_ANS: return 2700;
     default: return 6000;
     }
 }
