@@ -391,7 +391,11 @@ zf_status zf_mlp_adam(zf_mlp* net, const float* d_grad, float lr, void* stream);
  * mean loss of each epoch.  The inputs are standardized as (x - mean) / std
  * per feature, with the mean and standard deviation of these rows (std 1 for
  * a constant feature); the network keeps them and zf_mlp_predict and the
- * learned selector of zf_plan apply them (zf_mlp_get_scaling reads them). */
+ * learned selector of zf_plan apply them (zf_mlp_get_scaling reads them).
+ * The device memory for a call's rows is kept for the next zf_mlp_train or
+ * zf_mlp_predict of the network where it is at most 64 MB, and given back by
+ * zf_mlp_destroy; larger calls give theirs back before they return.  Calls of
+ * the two on one network wait for one another. */
 zf_status zf_mlp_train(zf_mlp* net, const float* h_x, const int32_t* h_y, const uint8_t* h_mask, uint32_t count,
                        uint32_t epochs, uint32_t batch, float lr, uint64_t seed, float* h_losses);
 /* Class of each host row (argmax of the logits over its allowed classes, -1

@@ -44,8 +44,8 @@ namespace {
 // block of text: 40% of them to parse, place and store tokens, the rest in
 // about equal parts shortcuts with lookups of bytes.  Measured on GB300: 21
 // blocks of text (1.3 MB) 85 us per call with its host part, 548 us with one
-// warp per block; 1,024 blocks 368 and 681 us.  Shortcuts whose steps were not
-// left for other tokens cost 27 us more of the 368.
+// warp per block; 1,024 blocks 333 and 652 us.  Shortcuts whose steps were not
+// left for other tokens cost 27 us more of them.
 constexpr uint32_t kLzThreads = 512;
 constexpr uint32_t kLzWarps = kLzThreads / 32;
 constexpr uint32_t kLzRing = 4096;             // parsed lengths: at most 1,023 left over and 2,048 more

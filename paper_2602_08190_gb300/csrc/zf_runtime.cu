@@ -13,7 +13,8 @@
 // may run at once (stages are independent): a launch too small to fill the
 // GPU -- an LZ77 stage has one CTA or warp per 64 KiB block -- overlaps the next.
 // The compute stream joins every decode stream at the end.  All descriptors
-// of a call are built on the host and copied once, ahead of the first stage.
+// of a call are built on the host; they travel as kernel parameters, or, where
+// a launch has too many, are copied once, ahead of the first stage.
 #include <cuda_runtime.h>
 
 #include <algorithm>
