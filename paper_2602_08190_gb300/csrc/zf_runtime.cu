@@ -323,6 +323,7 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         uint32_t dict_bytes = 0, lz_runs = 0;
     };
     std::vector<Key> keys;
+    const size_t g0 = groups.size();
     std::vector<uint8_t> key_of(e - b);   // a call has few groups: at most one per scheme and type
     for (size_t i = b; i < e; i++) {
         const zf::ChunkInfo& ch = *w[i].ch;
@@ -367,6 +368,10 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         }
         if (g.count) groups.push_back(g);
     }
+    // LZ77 and ANS first: their CTAs are few and slow, and a launch that fills the GPU keeps those behind it waiting
+    // (seven columns of 3M rows, one of them ANS, batched: 140 us with the batched launch first, 70 so)
+    std::stable_partition(groups.begin() + g0, groups.end(),
+                          [](const Group& g) { return g.scheme == ZF_LZ77 || g.scheme == ZF_ANS; });
 }
 
 // Whether every launch of a call takes its descriptors as parameters, so
