@@ -163,7 +163,8 @@ Geometry group_geometry(const zf_ctx* ctx, const zf_kcfg& k, int scheme, int dty
         else if (per_sm > 4096ull * at_once && per_sm < 4096ull * 32) g.tile_rows = 2048;
         return g;
     }
-    while (units && g.tile_rows > 1024 && per_sm < (uint64_t)g.tile_rows * 32) g.tile_rows /= 2;
+    // (string dictionaries through L1: 96 MB of 40,000 words take 242 us in whole jobs, 265 halved once, 246 in jobs of one tile)
+    while (units && g.tile_rows > 1024 && per_sm < (uint64_t)g.tile_rows * 32) g.tile_rows = scheme == ZF_STRDICT ? 1024 : g.tile_rows / 2;
     return g;
 }
 
@@ -280,22 +281,27 @@ constexpr int kStrdictSmem = ZF_NSCHEMES;
 
 bool fits_shared(const zf::ChunkInfo& ch) { return ch.scheme == ZF_STRDICT && ch.dict_bytes <= zf::strdict_smem_limit(); }
 
-// Whether the dictionaries of works[b, e) that fit go to shared memory.  A CTA
+// Whether the dictionaries of a call that fit go to shared memory.  A CTA
 // lays a chunk's dictionary out with its 32 warps waiting (about 15 us), then
 // each takes a tile: where an SM gets many chunks of few tiles that wait is
-// what a launch takes.  Text of 5,000 words in chunks of 64 KiB (11 tiles),
+// what a launch takes (for all stages of a call alike: a CTA of the one kernel
+// waits for an SM that CTAs of the other have left).  Text of 5,000 words in chunks of 64 KiB (11 tiles),
 // through L1 and with shared memory: 1.3 MB 57 and 47 us, 16 MB 111 and 75,
 // 64 MB (6.7 chunks per SM) 169 and 181, 256 MB 519 and 602; in chunks of 128
-// KiB (22 tiles) 56 and 36, 108 and 59, 156 and 130, 455 and 365.
+// KiB (22 tiles) 56 and 36, 108 and 59, 156 and 130, 455 and 365.  Chunks of
+// a tile or two (tokens of 64 bytes) do not pay for more than one dictionary:
+// the transfer of 48 MB of 500 such words in chunks of 64 KiB takes 378 us
+// through L1, 590 where stages of up to four chunks per SM took shared memory.
 constexpr uint32_t kShortChunkTiles = 16, kShortChunksPerSm = 4;
-bool strdict_shared(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_t e) {
+bool strdict_shared(const zf_ctx* ctx, const std::vector<Work>& works) {
     uint64_t n = 0, tiles = 0;
-    for (size_t i = b; i < e; i++)
-        if (fits_shared(*w[i].ch)) {
+    for (const Work& w : works)
+        if (fits_shared(*w.ch)) {
             n++;
-            tiles += (w[i].ch->units + zf::kStrTile - 1) / zf::kStrTile;
+            tiles += (w.ch->units + zf::kStrTile - 1) / zf::kStrTile;
         }
-    return tiles >= n * kShortChunkTiles || n <= (uint64_t)ctx->num_sms * kShortChunksPerSm;
+    return tiles >= n * kShortChunkTiles || n <= (uint64_t)ctx->num_sms ||
+           (2 * tiles >= n * kShortChunkTiles && n <= (uint64_t)ctx->num_sms * kShortChunksPerSm);
 }
 
 // The launch a chunk belongs to: LZ77, ANS and string dictionaries in shared
@@ -312,9 +318,9 @@ std::pair<int, int> group_key(const zf::ChunkInfo& ch, bool batched, bool shared
 // Append descriptors of works[b, e) to `desc`, grouped for launching.  A call
 // of 2,048 chunks (134M rows of FOR) took 189 us while a key was worked out
 // three times per chunk and the vectors grew as they filled; it takes 185.
-void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_t e, const zf_kcfg& k,
+void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_t e, bool shared, const zf_kcfg& k,
                   std::vector<ZfDevChunk>& desc, std::vector<Group>& groups) {
-    const bool batched = k.flags & ZF_KCFG_BATCHED, shared = strdict_shared(ctx, w, b, e);
+    const bool batched = k.flags & ZF_KCFG_BATCHED;
     struct Key {
         std::pair<int, int> key;
         uint32_t bmax = 0;         // widest bit width of the group: its geometry class
@@ -764,7 +770,9 @@ zf_status zf_transfer_decompress(zf_ctx* ctx, const zf_compressed* const* cols, 
     std::vector<ZfDevChunk> desc;
     desc.reserve(work.size());
     std::vector<std::vector<Group>> groups(stages.size());
-    for (size_t s = 0; s < stages.size(); s++) build_groups(ctx, work, stages[s].first, stages[s].second, k, desc, groups[s]);
+    const bool shared = strdict_shared(ctx, work);
+    for (size_t s = 0; s < stages.size(); s++)
+        build_groups(ctx, work, stages[s].first, stages[s].second, shared, k, desc, groups[s]);
     const size_t nd = std::max<size_t>(desc.size(), 1);
     ZfDevChunk* d_desc = nullptr;
     ZfDevChunk* h_desc = nullptr;
@@ -1007,7 +1015,7 @@ zf_status zf_decompress_resident(zf_ctx* ctx, const zf_resident* const* cols, ui
     std::vector<ZfDevChunk> desc;
     desc.reserve(work.size());
     std::vector<Group> groups;
-    build_groups(ctx, work, 0, work.size(), k, desc, groups);
+    build_groups(ctx, work, 0, work.size(), strdict_shared(ctx, work), k, desc, groups);
     ZF_CU(ctx, cudaEventRecord(ctx->ev_t0, ctx->compute));
     const bool inl = all_inline(groups);
     const bool same = inl || (desc.size() == ctx->resident_cache.size() &&

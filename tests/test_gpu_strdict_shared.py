@@ -37,6 +37,7 @@ CASES = {
     "1,025 entries": lambda: (_text(11, _words(11, 1025, 6, 8), 40_000), 1 << 20),
     "few short chunks": lambda: (_text(17, _words(17, 900, 3, 12), 4_500_000), 65536),
     "many short chunks": lambda: (_text(18, _words(18, 900, 3, 12), 6_500_000), 65536),
+    "chunks of one tile": lambda: (_text(19, _words(19, 500, 64, 64), 300_000), 65536),
     "CTA ranges across many chunks": lambda: (_text(12, _words(12, 3000, 3, 12), 900_000), 65536),
     "one chunk over all CTAs": lambda: (_text(13, _words(13, 5000, 3, 12), 500_000), 1 << 23),
     "dictionaries at the shared-memory limit": lambda: (_text(14, _words(14, 13_000, 6, 9), 300_000), 1 << 19),
