@@ -144,7 +144,7 @@ struct Geometry {
 // other schemes too are halved: a fact table of 16 columns of 0.7M rows, two
 // thirds of them FOR and dictionaries, takes 43 us, 48 with whole jobs.)
 Geometry group_geometry(const zf_ctx* ctx, const zf_kcfg& k, int scheme, int dtype, uint32_t bmax, uint64_t units,
-                        uint64_t short_tiled) {
+                        uint64_t short_tiled, bool tokens) {
     Geometry g{k.tile_rows, k.threads};
     if (scheme >= 0 && scheme < ZF_NSCHEMES && dtype >= 0 && dtype < 4) {
         const auto& t = ctx->tuned[scheme][dtype][width_bucket(bmax)];
@@ -163,8 +163,9 @@ Geometry group_geometry(const zf_ctx* ctx, const zf_kcfg& k, int scheme, int dty
         else if (per_sm > 4096ull * at_once && per_sm < 4096ull * 32) g.tile_rows = 2048;
         return g;
     }
-    // (string dictionaries through L1: 96 MB of 40,000 words take 242 us in whole jobs, 265 halved once, 246 in jobs of one tile)
-    while (units && g.tile_rows > 1024 && per_sm < (uint64_t)g.tile_rows * 32) g.tile_rows = scheme == ZF_STRDICT ? 1024 : g.tile_rows / 2;
+    // (string dictionaries through L1: 96 MB of 40,000 words take 242 us in whole jobs, 265 halved once, 246 in jobs of one
+    // tile; two columns of 40 MB in a batched launch 160, 191 and 150)
+    while (units && g.tile_rows > 1024 && per_sm < (uint64_t)g.tile_rows * 32) g.tile_rows = tokens ? 1024 : g.tile_rows / 2;
     return g;
 }
 
@@ -326,6 +327,7 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         uint32_t bmax = 0;         // widest bit width of the group: its geometry class
         uint64_t units = 0;        // rows (string dictionary: tokens) of the group
         uint64_t short_tiled = 0;  // those of FOR and dictionary chunks
+        bool tokens = false;       // whether string dictionaries are among them
         uint32_t dict_bytes = 0, lz_runs = 0;
     };
     std::vector<Key> keys;
@@ -340,6 +342,7 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         key_of[i - b] = (uint8_t)q;
         if (key.first >= 0) keys[q].bmax = std::max<uint32_t>(keys[q].bmax, ch.bmax);
         keys[q].units += ch.scheme == ZF_STRDICT ? ch.units : ch.rows;
+        keys[q].tokens |= ch.scheme == ZF_STRDICT;
         if (ch.scheme == ZF_FOR_BP || ch.scheme == ZF_DICT_BP) keys[q].short_tiled += ch.rows;
         keys[q].dict_bytes = std::max(keys[q].dict_bytes, ch.dict_bytes);
         keys[q].lz_runs += ch.lz_runs;
@@ -349,7 +352,7 @@ void build_groups(const zf_ctx* ctx, const std::vector<Work>& w, size_t b, size_
         const auto& key = kq.key;
         const Geometry geo = key.first == kStrdictSmem ? Geometry{zf::kStrTile, 0}
                                                        : group_geometry(ctx, k, key.first, key.second, kq.bmax, kq.units,
-                                                                        kq.short_tiled);
+                                                                        kq.short_tiled, kq.tokens);
         Group g{key.first, key.second, (uint32_t)desc.size(), 0, 0, 16, geo.tile_rows, geo.threads, kq.dict_bytes,
                 kq.lz_runs};
         for (size_t i = b; i < e; i++) {
@@ -1427,7 +1430,7 @@ extern "C" zf_status zf_ctx_tuned_geometry(const zf_ctx* ctx, int32_t scheme, in
     if (!ctx || !out || scheme < 0 || scheme >= ZF_NSCHEMES || dtype < 0 || dtype > ZF_F64 || bmax > 64)
         return ZF_EINVAL;
     const zf_kcfg k = effective_kcfg(ctx);
-    const Geometry g = group_geometry(ctx, k, scheme, dtype, bmax, 0, 0);
+    const Geometry g = group_geometry(ctx, k, scheme, dtype, bmax, 0, 0, false);
     *out = k;
     out->tile_rows = g.tile_rows;
     out->threads = g.threads;
