@@ -148,9 +148,9 @@ typedef struct {
                                  dictionary launches: 1024 below 8 and 14, 2048 while
                                  more than run at once but fewer than 32); LZ77, ANS and
                                  string dictionaries that fit in shared memory (without
-                                 ZF_KCFG_BATCHED; not launches of many chunks of under
-                                 16,384 tokens) have fixed jobs and read neither this
-                                 nor threads */
+                                 ZF_KCFG_BATCHED; not calls of many chunks of under
+                                 16,384 tokens or of many small stages) have fixed jobs
+                                 and read neither this nor threads */
     uint32_t threads;         /* 128, 256 or 512 (0 = the class's tuned value, else 128) */
     uint32_t ctas_per_sm;     /* batched launch: persistent grid = ctas_per_sm x SM count (0 = occupancy limit) */
     uint32_t stage_bytes;     /* pipeline stage: compressed bytes per H2D copy + decode step (default 64 MiB) */

@@ -293,14 +293,23 @@ bool fits_shared(const zf::ChunkInfo& ch) { return ch.scheme == ZF_STRDICT && ch
 // a tile or two (tokens of 64 bytes) do not pay for more than one dictionary:
 // the transfer of 48 MB of 500 such words in chunks of 64 KiB takes 378 us
 // through L1, 590 where stages of up to four chunks per SM took shared memory.
-constexpr uint32_t kShortChunkTiles = 16, kShortChunksPerSm = 4;
-bool strdict_shared(const zf_ctx* ctx, const std::vector<Work>& works) {
-    uint64_t n = 0, tiles = 0;
-    for (const Work& w : works)
-        if (fits_shared(*w.ch)) {
-            n++;
-            tiles += (w.ch->units + zf::kStrTile - 1) / zf::kStrTile;
-        }
+// And each stage's launch takes every SM, one after the other, where several
+// of the L1 kernel run at once: 256 MB in 4 MB chunks and stages of 2, 4, 8 and
+// 64 MiB take 1,159, 627, 532 and 614 us through L1, 1,779, 722, 454 and 498
+// with shared memory, so a row of small stages stays with L1.
+constexpr uint32_t kShortChunkTiles = 16, kShortChunksPerSm = 4, kSmallStageTilesPerSm = 20, kSmallStages = 8;
+bool strdict_shared(const zf_ctx* ctx, const std::vector<Work>& works, const std::vector<std::pair<size_t, size_t>>& stages) {
+    uint64_t n = 0, tiles = 0, in = 0;   // chunks, their tiles, stages that hold some
+    for (const auto& s : stages) {
+        const uint64_t before = n;
+        for (size_t i = s.first; i < s.second; i++)
+            if (fits_shared(*works[i].ch)) {
+                n++;
+                tiles += (works[i].ch->units + zf::kStrTile - 1) / zf::kStrTile;
+            }
+        in += n > before;
+    }
+    if (in >= kSmallStages && tiles < in * ctx->num_sms * kSmallStageTilesPerSm) return false;
     return tiles >= n * kShortChunkTiles || n <= (uint64_t)ctx->num_sms ||
            (2 * tiles >= n * kShortChunkTiles && n <= (uint64_t)ctx->num_sms * kShortChunksPerSm);
 }
@@ -773,7 +782,7 @@ zf_status zf_transfer_decompress(zf_ctx* ctx, const zf_compressed* const* cols, 
     std::vector<ZfDevChunk> desc;
     desc.reserve(work.size());
     std::vector<std::vector<Group>> groups(stages.size());
-    const bool shared = strdict_shared(ctx, work);
+    const bool shared = strdict_shared(ctx, work, stages);
     for (size_t s = 0; s < stages.size(); s++)
         build_groups(ctx, work, stages[s].first, stages[s].second, shared, k, desc, groups[s]);
     const size_t nd = std::max<size_t>(desc.size(), 1);
@@ -1018,7 +1027,7 @@ zf_status zf_decompress_resident(zf_ctx* ctx, const zf_resident* const* cols, ui
     std::vector<ZfDevChunk> desc;
     desc.reserve(work.size());
     std::vector<Group> groups;
-    build_groups(ctx, work, 0, work.size(), strdict_shared(ctx, work), k, desc, groups);
+    build_groups(ctx, work, 0, work.size(), strdict_shared(ctx, work, {{0, work.size()}}), k, desc, groups);
     ZF_CU(ctx, cudaEventRecord(ctx->ev_t0, ctx->compute));
     const bool inl = all_inline(groups);
     const bool same = inl || (desc.size() == ctx->resident_cache.size() &&

@@ -2,10 +2,11 @@
 batches (64 tokens), tiles (1024 tokens), dictionaries and CTA ranges begin and
 end, columns whose chunks take both kernels (dictionaries that fit in shared
 memory and ones that do not), and short chunks on either side of the four per
-SM (608 on 152 SMs) from which a launch reads them through L1."""
+SM (608 on 152 SMs) from which a call reads them through L1."""
 import numpy as np
 import pytest
 
+import zf_workloads as W
 from gpu_helpers import Gpu, out_specs
 
 zf = pytest.importorskip("paper_2602_08190_gb300")
@@ -82,6 +83,22 @@ def test_warps_of_several_tiles(lo, hi, tokens):
         for _ in range(3):
             got_t, got_o = g.decode([h], out_specs(t, o), resident=True)
             assert np.array_equal(got_t, t) and np.array_equal(got_o, o)
+    finally:
+        zf.zf_compressed_free(h)
+        g.close()
+
+
+# Eight stages and more of few tiles each are decoded through L1, fewer or
+# larger ones with the dictionary in shared memory.
+@pytest.mark.parametrize("stage_mib", [1, 2, 64])
+def test_stages(stage_mib):
+    t, o = W.text_column(3, 48 << 20)
+    col = zf.Column(t, o)
+    h = zf.zf_compress_host(zf.zf_plan(None, col, scheme=zf.ZF_STRDICT, chunk_rows=1 << 20), col)
+    g = Gpu(stage_bytes=stage_mib << 20)
+    try:
+        got_t, got_o = g.decode([h], out_specs(t, o))
+        assert np.array_equal(got_t, t) and np.array_equal(got_o, o)
     finally:
         zf.zf_compressed_free(h)
         g.close()
