@@ -42,10 +42,10 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 // Launches of at most this many blocks per SM take a CTA per block
 // (zf_lz_cta.cu).  A warp takes 500 us for a block of text however few there
 // are, a CTA per block adds 0.3 us for each block to about 60 us: resident
-// calls of 16, 64 and 130 MB of text take 108, 333 and 625 us with a CTA and
-// 556, 652 and 770 us with a warp per block, and at 19 blocks per SM they would
+// calls of 16, 64 and 130 MB of text take 102, 327 and 601 us with a CTA and
+// 556, 652 and 770 us with a warp per block, and at 20 blocks per SM they would
 // be even.  130 MB (13.7 per SM) of zeros take 442 and 473, of int32 values below
-// 1,000 910 and 943, which are even at 15.
+// 1,000 944 and 943.
 // Blocks of long literal runs between long matches (fields padded with blanks)
 // leave the warp kernel little to parse and the CTA kernel literals that its
 // ring does not hold: 64 and 130 MB took 331 and 605 us with a CTA, 414 and 495

@@ -24,7 +24,8 @@ namespace {
 //   it, so a byte finds its token by one popcount.
 //   Shortcuts: a match whose source lies inside one earlier match of the
 //   segment copies that match's source instead (the offsets add up), again
-//   until its source is no match or lies before the segment: a word's earlier
+//   until its source is no match or lies before the segment, a few times at
+//   the most: a word's earlier
 //   occurrences form chains of 11 copies for the longest of 128 bytes of text,
 //   3 after this.
 //   Bytes: thread i takes the segment's aligned 4-byte words i, i + 512, ...: a
@@ -43,8 +44,8 @@ namespace {
 // blocks it is bound by issue slots (64% busy), 229,000 warp instructions per
 // block of text: 40% of them to parse, place and store tokens, the rest in
 // about equal parts shortcuts with lookups of bytes.  Measured on GB300: 21
-// blocks of text (1.3 MB) 85 us per call with its host part, 548 us with one
-// warp per block; 1,024 blocks 333 and 652 us.  Shortcuts whose steps were not
+// blocks of text (1.3 MB) 82 us per call with its host part, 548 us with one
+// warp per block; 1,024 blocks 327 and 652 us.  Shortcuts whose steps were not
 // left for other tokens cost 27 us more of them.
 constexpr uint32_t kLzThreads = 512;
 constexpr uint32_t kLzWarps = kLzThreads / 32;
@@ -52,6 +53,11 @@ constexpr uint32_t kLzRing = 4096;             // parsed lengths: at most 1,023 
 constexpr uint32_t kLzStep = 4 * kLzThreads;   // bytes of the lengths stream parsed per step
 constexpr uint32_t kLzSeg = 8192;              // output bytes of a segment, from its first aligned word
 constexpr uint32_t kLzLit = 8192;              // ring of literal bytes
+// Shortcut steps of a token.  A match that overlaps its own output (a run) is
+// left period by period: without a bound, 512 random bytes and 512 zeros in turn
+// took 655 us a block, where the bytes' own way into the run's first period is
+// one step.  120 MB of text: 554 us with 4, 579 with 8, 16 or no bound.
+constexpr uint32_t kLzShortcuts = 4;
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kDone = 0x8000u;            // state of a byte: kDone | value, or the position it copies
 
@@ -303,19 +309,18 @@ __device__ void lz_block(const ZfDevChunk& c, LzSmem& sm, uint32_t* err) {
             if (__syncthreads_or(bad)) { ok = false; break; }
             if (has_m && mpos < s1 && oend > s0) {
                 // the source lies inside one match of this segment: copy what that match copies; every step is
-                // left for the tokens that look here, so a chain of n matches takes about log2 n steps
+                // left for the tokens that look here, so a chain of n matches takes about log2 n steps, and what is
+                // left of it the bytes follow by themselves
                 uint32_t o = off;
-                for (;;) {
+#pragma unroll 1
+                for (uint32_t step = 0; step < kLzShortcuts; step++) {
                     const uint32_t src = mpos - o;
                     if (src < s0 || o < ml) break;
                     const uint32_t n = lz_token(sm.starts[(src - base) >> 5], (src - base) & 31u);
                     const uint2* u = &sm.tok[n ? n - 1 : 0];
                     const uint32_t ux = *const_cast<const volatile uint32_t*>(&u->x);   // its owner may shorten it meanwhile
                     if (src <= (ux & 0xFFFFu) || src + ml - 1 > (u->y >> 16)) break;
-                    // a match that overlaps its own output (a run): into its first period at once, not period by period
-                    const uint32_t uo = ux >> 16, d = src - 1 - (ux & 0xFFFFu);
-                    o += uo;
-                    if (d >= uo) o += d / uo * uo;
+                    o += ux >> 16;
                     *reinterpret_cast<volatile uint32_t*>(&sm.tok[tid].x) = (mpos - 1) | (o << 16);
                 }
             }
